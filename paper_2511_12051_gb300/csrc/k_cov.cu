@@ -424,50 +424,68 @@ static int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // Shared-memory passes of one warp's two load instructions (row block and
 // column block of a look) in the pixel-major buffer: per half-warp, the
 // largest number of distinct 8-byte words that share one of 16 banks.  The
-// lanes are laid out as in cov_tile; its PPW pixels sit sy * pitch pixels apart.
-static int bank_passes(int B, int BN, int S, int sy, int pitch) {
+// lanes are laid out as in cov_tile; its PPW pixels sit `stride` dates apart
+// (sy * pitch * S), of which only stride mod 16 moves a bank: a pixel is
+// farther from the next than any two dates of one pixel, so words of
+// different pixels never coincide.
+static constexpr int bank_passes(int B, int BN, int stride) {
     const int U = BN * (BN + 1) / 2, PPW = 32 / U;
-    int lane_slot[32], lane_bi[32], lane_bk[32];
-    for (int lane = 0; lane < 32; ++lane) {
-        int gs = lane / U, u = lane - gs * U;
-        if (gs >= PPW) {
-            gs = PPW - 1;
-            u = lane - PPW * U;
-        }
-        int bi = 0, bk = 0, t = u;
-        for (int a = 0; a < BN; ++a) {
-            const int len = BN - a;
-            if (t >= 0 && t < len) { bi = a; bk = a + t; }
-            t -= len;
-        }
-        lane_slot[lane] = gs;
-        lane_bi[lane] = bi;
-        lane_bk[lane] = bk;
-    }
     int total = 0;
     for (int which = 0; which < 2; ++which)
         for (int half = 0; half < 2; ++half) {
-            long long addr[16];
-            int na = 0;
+            int slot[16] = {}, word[16] = {}, na = 0, per_bank[16] = {}, worst = 0;
             for (int l = half * 16; l < half * 16 + 16; ++l) {
-                const long long a =
-                    (long long)lane_slot[l] * sy * pitch * S + (long long)(which ? lane_bk[l] : lane_bi[l]) * B;
+                int gs = l / U, u = l - gs * U;
+                if (gs >= PPW) {
+                    gs = PPW - 1;
+                    u = l - PPW * U;
+                }
+                int bi = 0, bk = 0, t = u;
+                for (int a = 0; a < BN; ++a) {
+                    const int len = BN - a;
+                    if (t >= 0 && t < len) {
+                        bi = a;
+                        bk = a + t;
+                    }
+                    t -= len;
+                }
+                const int w = (which ? bk : bi) * B;
                 bool seen = false;
-                for (int j = 0; j < na; ++j) seen = seen || addr[j] == a;
-                if (!seen) addr[na++] = a;
+                for (int j = 0; j < na; ++j) seen = seen || (slot[j] == gs && word[j] == w);
+                if (seen) continue;
+                slot[na] = gs;
+                word[na++] = w;
+                const int bank = (gs * stride + w) % 16;
+                ++per_bank[bank];
+                if (per_bank[bank] > worst) worst = per_bank[bank];
             }
-            int per_bank[16] = {0}, worst = 0;
-            for (int j = 0; j < na; ++j) worst = std::max(worst, ++per_bank[addr[j] % 16]);
             total += worst;
         }
     return total;
 }
 
+// bank_passes of every stride mod 16, counted by the compiler: the tile search
+// asks for up to sixteen pitches of its candidates, on every call, and counting
+// them there took 0.35 ms of host time, twice as long as the rest of a step of
+// a 128 x 128 stack (N = 10, stride 1: 0.52 ms a step, 0.17 ms with the table).
+struct PassTable {
+    int passes[16];
+};
+static constexpr PassTable make_pass_table(int B, int BN) {
+    PassTable t{};
+    for (int r = 0; r < 16; ++r) t.passes[r] = bank_passes(B, BN, r);
+    return t;
+}
+template <int B, int BN>
+struct BankPasses {
+    static constexpr PassTable table = make_pass_table(B, BN);
+};
+
 // Smallest row pitch >= rx with the fewest bank passes.
-static int row_pitch(int B, int BN, int S, int rx, int sy) {
+static int row_pitch(const PassTable &tab, int S, int rx, int sy) {
     int best = rx, best_cost = 1 << 30;
     for (int p = rx; p < rx + 16; ++p) {
-        const int c = bank_passes(B, BN, S, sy, p);
+        const int c = tab.passes[((unsigned)sy * (unsigned)p * (unsigned)S) & 15u];
         if (c < best_cost) {
             best_cost = c;
             best = p;
@@ -476,13 +494,13 @@ static int row_pitch(int B, int BN, int S, int rx, int sy) {
     return best;
 }
 
-static CovLayout make_layout(int n, int B, int BN, int S, const Geom &g, int TY, int TX) {
+static CovLayout make_layout(int n, const PassTable &tab, int S, const Geom &g, int TY, int TX) {
     CovLayout l{};
     l.TY = TY;
     l.TX = TX;
     l.RY = (TY - 1) * g.sy + g.wy;
     l.RX = round_up((TX - 1) * g.sx + g.wx + 1, 2);
-    l.RXc = row_pitch(B, BN, S, l.RX, g.sy);
+    l.RXc = row_pitch(tab, S, l.RX, g.sy);
     l.Z0 = round_up(l.RY * l.RXc, 16);
     l.PSs = round_up(l.RY * l.RX, 16);
     l.smem_plain = (size_t)(l.Z0 + 16) * S * sizeof(float2);
@@ -492,7 +510,7 @@ static CovLayout make_layout(int n, int B, int BN, int S, const Geom &g, int TY,
 
 // Tile choice: PPW pixels stacked per warp column, 8 warps, several passes for
 // small strides; the score favours full warps and little halo per output pixel.
-static CovLayout choose_layout(int n, int B, int BN, int S, const Geom &g, size_t budget, bool tma) {
+static CovLayout choose_layout(int n, const PassTable &tab, int BN, int S, const Geom &g, size_t budget, bool tma) {
     const int ppw = 32 / (BN * (BN + 1) / 2);
     CovLayout best{};
     double best_score = -1.0;
@@ -501,17 +519,17 @@ static CovLayout choose_layout(int n, int B, int BN, int S, const Geom &g, size_
             const int TY = ppw * a;
             const int px = TY * TX;
             if (px > 8 * ppw * 8) continue;
-            CovLayout l = make_layout(n, B, BN, S, g, TY, TX);
-            const size_t sm = tma ? l.smem_tma : l.smem_plain;
-            if (sm > budget || l.RX > 256 || l.RY > 256) continue;
-            const double halo = (double)(TY * g.sy) * (TX * g.sx) / ((double)l.RY * l.RX);
+            const int RY = (TY - 1) * g.sy + g.wy, RX = round_up((TX - 1) * g.sx + g.wx + 1, 2);
+            if (RX > 256 || RY > 256) continue;
+            const double halo = (double)(TY * g.sy) * (TX * g.sx) / ((double)RY * RX);
             const int per_pass = 8 * ppw;
             const double lane_eff = (double)px / (((px + per_pass - 1) / per_pass) * per_pass);
             const double score = lane_eff * (0.6 + 0.4 * halo);
-            if (score > best_score) {
-                best_score = score;
-                best = l;
-            }
+            if (!(score > best_score)) continue;
+            const CovLayout l = make_layout(n, tab, S, g, TY, TX);
+            if ((tma ? l.smem_tma : l.smem_plain) > budget) continue;
+            best_score = score;
+            best = l;
         }
     return best;
 }
@@ -527,6 +545,7 @@ static void block_shape(int n, int &B, int &BN) {
 int covariance_tile_candidates(int n, const Geom &g, int (*tiles)[2], int max) {
     int B, BN;
     block_shape(n, B, BN);
+    const PassTable tab = make_pass_table(B, BN);
     const int S = (B * BN) % 2 ? B * BN : B * BN + 1;
     const int ppw = 32 / (BN * (BN + 1) / 2);
     const size_t kHalfSm = 113 * 1024;
@@ -541,7 +560,7 @@ int covariance_tile_candidates(int n, const Geom &g, int (*tiles)[2], int max) {
             const int TY = ppw * a;
             const int px = TY * TX;
             if (px > 8 * ppw * 8) continue;
-            CovLayout l = make_layout(n, B, BN, S, g, TY, TX);
+            CovLayout l = make_layout(n, tab, S, g, TY, TX);
             if (l.smem_plain > kHalfSm) continue;
             const double halo = (double)(TY * g.sy) * (TX * g.sx) / ((double)l.RY * l.RX);
             const int per_pass = 8 * ppw;
@@ -561,6 +580,7 @@ template <int B, int BN>
 static cudaError_t run_cov(const Planes &z, int n, const Geom &g, const uint64_t *mask, float2 *C,
                            cudaStream_t s, const Schedule *sch) {
     constexpr int S = PixStride<B, BN>::value;
+    const PassTable &tab = BankPasses<B, BN>::table;
     const size_t kMaxSmem = 226 * 1024;
 #ifndef PLK_COV_NO_ASYNC
     {
@@ -569,10 +589,10 @@ static cudaError_t run_cov(const Planes &z, int n, const Geom &g, const uint64_t
         const size_t kHalfSm = 113 * 1024;
         CovLayout la{};
         if (sch && sch->cov_TY > 0 && sch->cov_TX > 0 && sch->cov_TY % (32 / (BN * (BN + 1) / 2)) == 0) {
-            la = make_layout(n, B, BN, S, g, sch->cov_TY, sch->cov_TX);
+            la = make_layout(n, tab, S, g, sch->cov_TY, sch->cov_TX);
             if (la.smem_plain > kHalfSm) la = CovLayout{};
         }
-        if (la.TY == 0) la = choose_layout(n, B, BN, S, g, kHalfSm, false);
+        if (la.TY == 0) la = choose_layout(n, tab, BN, S, g, kHalfSm, false);
         if (la.TY > 0) {
             cudaError_t e = cudaFuncSetAttribute(k_cov_async<B, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)kHalfSm);
@@ -591,7 +611,7 @@ static cudaError_t run_cov(const Planes &z, int n, const Geom &g, const uint64_t
         }
     }
 #endif
-    CovLayout lay = choose_layout(n, B, BN, S, g, kMaxSmem, true);
+    CovLayout lay = choose_layout(n, tab, BN, S, g, kMaxSmem, true);
     TmaMaps maps;
     if (lay.TY > 0 && encode_plane_maps(maps, z, n, g, lay.RX, lay.RY)) {
         cudaError_t e =
@@ -604,10 +624,10 @@ static cudaError_t run_cov(const Planes &z, int n, const Geom &g, const uint64_t
         k_cov_tma<B, BN><<<(unsigned)grid, 256, lay.smem_tma, s>>>(maps, n, g, mask, C, lay, ntiles, tilesY);
         return cudaGetLastError();
     }
-    lay = choose_layout(n, B, BN, S, g, 96 * 1024, false);
-    if (lay.TY == 0) lay = choose_layout(n, B, BN, S, g, kMaxSmem, false);
+    lay = choose_layout(n, tab, BN, S, g, 96 * 1024, false);
+    if (lay.TY == 0) lay = choose_layout(n, tab, BN, S, g, kMaxSmem, false);
     if (lay.TY == 0) {
-        lay = make_layout(n, B, BN, S, g, 1, 1);
+        lay = make_layout(n, tab, S, g, 1, 1);
         if (lay.smem_plain > kMaxSmem) return cudaErrorInvalidConfiguration;
     }
     cudaError_t e =
