@@ -21,6 +21,7 @@
 // Per input pixel q and date i (gather):  g_i(q) = sum over the output
 //   pixels p whose window holds q with the mask bit set of (H_p z(q))_i.
 #include <algorithm>
+#include <type_traits>
 
 #include "emi.cuh"
 
@@ -28,9 +29,7 @@ namespace plk {
 
 namespace {
 
-constexpr int kAdjWarps = 2;
-
-// Row of the coherence cached in shared memory, padded (see k_emi.cu).
+// Row of the coherence in shared memory, padded (see k_emi.cu).
 template <int NP>
 struct AdjRow {
     static constexpr bool kPadded = true;
@@ -46,13 +45,143 @@ struct AdjRow {
     }
 };
 
-// Publish every lane's row of an NP x NP matrix to the group's buffer.
-template <int NP, class S>
-__device__ __forceinline__ void publish(const S (&row)[NP], S *mat, int r, unsigned gmask) {
-    __syncwarp(gmask);
+// Two entries of a row, 16-byte aligned.
+__device__ __forceinline__ void load_pair(const cpx<float> *src, cpx<float> (&c)[2]) {
+    const float4 v = *reinterpret_cast<const float4 *>(src);
+    c[0] = mk<float>(v.x, v.y);
+    c[1] = mk<float>(v.z, v.w);
+}
+template <int NP>
+__device__ __forceinline__ void store_row(float *dst, const float (&row)[NP]) {
 #pragma unroll
-    for (int k = 0; k < NP; ++k) mat[r * NP + k] = row[k];
+    for (int k = 0; k < NP; k += 4)
+        *reinterpret_cast<float4 *>(dst + k) = make_float4(row[k], row[k + 1], row[k + 2], row[k + 3]);
+}
+
+// Shared memory of one group (output pixel), in bytes from its base.  C holds
+// NP padded rows and a zero row for the lanes past the last one (rows of 20,
+// 24 and 28 entries run one pixel a warp); its pitch of NP + 2 entries puts the
+// 16-byte chunks of 8 consecutive rows in different banks, and a row is also
+// read as a broadcast.  Matrices of one value a lane are stored [k][r] (entry
+// k of lane r's row), so a row's owner reads it without bank conflicts.
+template <int NP>
+struct AdjShared {
+    static constexpr bool kPow2 = (NP & (NP - 1)) == 0;
+    static constexpr int G = kPow2 ? 32 / NP : 1;
+    static constexpr int kPitch = NP + 2;
+    static constexpr int kLanes = kPow2 ? NP : 32;
+    static constexpr int kMat = NP * NP * 4;  // one float matrix
+    static constexpr int kBuf = (NP + 2 > kLanes ? NP + 2 : kLanes) * 8;
+    static constexpr int oC = 0;
+    static constexpr int oBuf = oC + (NP + 1) * kPitch * 8;
+    static constexpr int oV = oBuf + kBuf;
+    static constexpr int oRs = oV + kLanes * 8;
+    static constexpr int oM = oRs + kLanes * 4;  // two float matrices: the G^-1 row slots, then products
+    static constexpr int oG = oM + 2 * kMat;     // G^-1 [k][r]
+    static_assert(2 * kMat >= kLanes * (NP + 4) * 4, "the G^-1 row slots fit the product matrices");
+    static_assert(oM % 16 == 0 && kMat % 16 == 0, "16-byte loads");
+    char *base;
+    __device__ __forceinline__ cpx<float> *C() const { return reinterpret_cast<cpx<float> *>(base + oC); }
+    __device__ __forceinline__ cpx<float> *buf() const { return reinterpret_cast<cpx<float> *>(base + oBuf); }
+    __device__ __forceinline__ cpx<float> *v() const { return reinterpret_cast<cpx<float> *>(base + oV); }
+    __device__ __forceinline__ float *rs() const { return reinterpret_cast<float *>(base + oRs); }
+    __device__ __forceinline__ float *M() const { return reinterpret_cast<float *>(base + oM); }
+    __device__ __forceinline__ float *g() const { return reinterpret_cast<float *>(base + oG); }
+};
+
+// Lane numbering of a group.
+template <int NP>
+struct AdjLane {
+    int r, glane0, rr;  // row; first lane of the group; a row that exists (lanes past the last read it)
+    unsigned gmask;
+    __device__ __forceinline__ AdjLane(int lane) {
+        constexpr bool kPow2 = (NP & (NP - 1)) == 0;
+        const int grp = kPow2 ? lane / NP : 0;
+        r = lane - grp * NP;
+        rr = r < NP ? r : NP - 1;
+        glane0 = grp * NP;
+        gmask = (!kPow2 || NP == 32) ? 0xffffffffu : (((1u << NP) - 1u) << glane0);
+    }
+};
+
+// C <- the padded Hermitian matrix of the packed triangle: row i of the
+// triangle is read by consecutive lanes and written as row and column i.
+template <int NP>
+__device__ __forceinline__ void adj_load(const AdjShared<NP> &sh, const float2 *__restrict__ Cpix, int r, int n) {
+    constexpr int P = AdjShared<NP>::kPitch;
+    cpx<float> *C = sh.C();
+#pragma unroll 4
+    for (int i = 0; i < NP; ++i) {
+        if (r < i || r >= NP) continue;
+        float2 c = make_float2(i == r && i >= n ? 1.f : 0.f, 0.f);
+        if (r < n) c = __ldg(Cpix + packed_index(n, i, r));
+        C[i * P + r] = mk<float>(c.x, c.y);
+        if (r > i) C[r * P + i] = mk<float>(c.x, -c.y);
+    }
+    if (r < NP) C[NP * P + r] = mk<float>(0.f, 0.f);
+}
+
+// Per-pixel part of the adjoint: solves the pixel (v into shared memory), puts
+// G^-1 into shared memory (1 between live dates on the EVD fallback) and
+// leaves this lane's row of M = (A - lambda I + c v v^H)^-1 in mrow.  G^-1 is
+// the one that the solve leaves in its row slots.  Dates without power
+// (S_kk = 0) carry no gradient: their rows and columns of g are 0.
+template <int NP>
+struct AdjPixel {
+    cpx<float> v;
+    float rsr, cdef;
+    bool evd, live;
+};
+
+template <int NP>
+__device__ __forceinline__ void adj_prepare(AdjPixel<NP> &S, cpx<float> (&mrow)[NP], const AdjShared<NP> &sh,
+                                            const AdjLane<NP> &L, const float *__restrict__ Sd, long long p, int n,
+                                            int ref, const EmiParams &q) {
+    constexpr int P = AdjShared<NP>::kPitch;
+    const int r = L.r;
+    const unsigned gmask = L.gmask;
+    cpx<float> *cbuf = sh.buf();
+    const AdjRow<NP> ld{sh.C() + (r < NP ? r : NP) * P};
+    float *gslot = sh.M() + r * (NP + 4);
+    S.live = r < n;
+    const PixelResult res =
+        emi_solve<NP, float, AdjRow<NP>, true>(ld, r, n, ref, q, cbuf, gmask, L.glane0, false, gslot);
+    S.evd = res.evd;
+    S.v = S.live ? res.v : mk<float>(0.f, 0.f);
+    const float sr = S.live ? __ldg(Sd + p * n + r) : 0.f;
+    S.rsr = sr > 0.f ? rsqrtf(sr) : 0.f;
+    sh.v()[r] = S.v;
+    sh.rs()[r] = S.rsr;
     __syncwarp(gmask);
+    // A row (C, or G^-1 o C) into mrow, the masked G^-1 row into [k][r].
+    ld.all(mrow);
+#pragma unroll
+    for (int q4 = 0; q4 < NP / 4; ++q4) {
+        const float4 g4 = reinterpret_cast<const float4 *>(gslot)[q4];
+        const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int k = q4 * 4 + e;
+            const float gk = S.evd ? 1.f : gg[e];
+            mrow[k] = mk<float>(gk * mrow[k].x, gk * mrow[k].y);
+            if (r < NP) sh.g()[k * NP + r] = S.rsr > 0.f && sh.rs()[k] > 0.f ? gk : 0.f;
+        }
+    }
+    // lambda = v^H A v (the eigenvalue the perturbation is about)
+    const cpx<float> av = group_matvec<NP, float>(mrow, S.v, cbuf, r, gmask);
+    const float lam = group_sum<NP, float>(S.live ? (S.v.x * av.x + S.v.y * av.y) : 0.f, gmask);
+    // c keeps the deflated matrix well scaled, with the sign that leaves it
+    // definite (A - lambda I is positive semidefinite, on the EVD fallback
+    // negative: lambda is the largest eigenvalue of C), so that the inversion
+    // without pivoting meets no zero pivot (a single look and four dates did)
+    S.cdef = S.evd ? -fmaxf(1.f, fabsf(lam)) : fmaxf(1.f, fabsf(lam));
+    const cpx<float> cv = S.cdef * S.v;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        mrow[k] = mrow[k] + cv * conj(sh.v()[k]);
+        if (k == r && S.live) mrow[k].x -= lam;
+    }
+    gj_invert<NP, float, cpx<float>, false>(mrow, cbuf, r, n, gmask, 0.f);
 }
 
 }  // namespace
@@ -82,220 +211,41 @@ __global__ void __launch_bounds__(256) k_adj_sdiag(const __grid_constant__ Plane
     }
 }
 
-// Per-pixel state of the uncertainty kernel that does not depend on the date:
-// in registers, this lane's eigenvector entry and its row of the inverted
-// deflated matrix (A - lambda I + c v v^H)^-1; in the group's shared memory
-// (UncShared), the coherence row (the lane's row cache), every lane's v, every
-// 1/sqrt(S_kk) and G^-1.  Keeping the group-uniform vectors and the rows that
-// are only read out of the register file leaves the per-date products room.
-template <int NP>
-struct AdjPixelState {
-    cpx<float> v, mrow[NP];
-    float sr, rsr;
-    bool evd, live;
-};
-
-// Group views of the shared buffers: row r of C (myrow, padded), v and
-// 1/sqrt(S_kk) of every lane, G^-1 [NP][NP].
-template <int NP>
-struct UncShared {
-    const cpx<float> *myrow;
-    cpx<float> *vg;
-    float *rsg;
-    float *ginv;
-};
-
-template <int NP>
-__device__ __forceinline__ void adj_prepare(AdjPixelState<NP> &S, const UncShared<NP> &sh, const float *__restrict__ Sd,
-                                            long long p, int r, int n, int ref, const EmiParams &q,
-                                            cpx<float> *cbuf, unsigned gmask, int glane0) {
-    float *rbuf = reinterpret_cast<float *>(cbuf);
-    const AdjRow<NP> ld{sh.myrow};
-    S.live = r < n;
-    const PixelResult res = emi_solve<NP, float>(ld, r, n, ref, q, cbuf, gmask, glane0, false);
-    S.evd = res.evd;
-    S.v = S.live ? res.v : mk<float>(0.f, 0.f);
-    // G^-1 row, published to the group's matrix.
-    {
-        float gi[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            float m = mag_t(norm2(sh.myrow[k]));
-            if (q.beta != 0.f) m = (1.f - q.beta) * m + ((k == r) ? q.beta : 0.f);
-            gi[k] = m;
-        }
-        if (!S.evd) gj_invert<NP, float, float, true>(gi, rbuf, r, n, gmask, 0.f);
-        publish<NP, float>(gi, sh.ginv, r, gmask);
-    }
-    // A row (C, or G^-1 o C) into mrow; lambda = v^H A v.
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const cpx<float> c = sh.myrow[k];
-        const float gk = sh.ginv[r * NP + k];
-        S.mrow[k] = S.evd ? c : mk<float>(gk * c.x, gk * c.y);
-    }
-    const cpx<float> av = group_matvec<NP, float>(S.mrow, S.v, cbuf, r, gmask);
-    const float lam = group_sum<NP, float>(S.live ? (S.v.x * av.x + S.v.y * av.y) : 0.f, gmask);
-    sh.vg[r] = S.v;
-    __syncwarp(gmask);
-    // (A - lambda I + c v v^H)^-1  (c keeps the deflated matrix well scaled)
-    const float cdef = fmaxf(1.f, fabsf(lam));
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        S.mrow[k] = S.mrow[k] + cdef * (S.v * conj(sh.vg[k]));
-        if (k == r && S.live) S.mrow[k].x -= lam;
-    }
-    gj_invert<NP, float, cpx<float>, false>(S.mrow, cbuf, r, n, gmask, 0.f);
-    S.sr = S.live ? __ldg(Sd + p * n + r) : 0.f;
-    S.rsr = S.sr > 0.f ? rsqrtf(S.sr) : 0.f;
-    sh.rsg[r] = S.rsr;
-    __syncwarp(gmask);
-}
-
-// Row r of H = GS + GS^H for the phase weight wr of this lane's date (the
-// weight of the reference date is unused: its phase is 0).  Products over the
-// date index stop at n (rows and columns past n are zero).
-template <int NP>
-__device__ __forceinline__ void adj_h_row(const AdjPixelState<NP> &S, const UncShared<NP> &sh, float wr, int r, int n,
-                                          int ref, float beta, cpx<float> *cbuf, cpx<float> *cmat, unsigned gmask,
-                                          cpx<float> (&h)[NP]) {
-    float *fmat = reinterpret_cast<float *>(cmat);
-    // Gradient on v (gauge-free), projected orthogonal to v.
-    const float wsum = group_sum<NP, float>(S.live && r != ref ? wr : 0.f, gmask);
-    const float m2 = norm2(S.v);
-    const float coef = (r == ref) ? -wsum : wr;
-    cpx<float> gv = (S.live && m2 > 0.f) ? (coef / m2) * mk<float>(-S.v.y, S.v.x) : mk<float>(0.f, 0.f);
-    {
-        const cpx<float> t = conj(S.v) * gv;
-        const float sx = group_sum<NP, float>(t.x, gmask), sy = group_sum<NP, float>(t.y, gmask);
-        gv = gv - S.v * mk<float>(sx, sy);
-    }
-    // u = (A - lambda I + c v v^H)^-1 g_v  (u orthogonal to v)
-    const cpx<float> u = group_matvec<NP, float>(S.mrow, gv, cbuf, r, gmask);
-
-    // GA = -u v^H (row r), then GC (off the diagonal); h holds GC.
-#pragma unroll
-    for (int k = 0; k < NP; ++k) h[k] = mk<float>(0.f, 0.f) - u * conj(sh.vg[k]);
-    if (!S.evd) {
-        float T[NP];
-        {
-            float R[NP];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const cpx<float> c = sh.myrow[k];
-                R[k] = h[k].x * c.x + h[k].y * c.y;  // Re(conj(GA) C)
-            }
-            publish<NP, float>(R, fmat, r, gmask);
-        }
-        // T = G^-1 R (row r)
-#pragma unroll
-        for (int k = 0; k < NP; ++k) T[k] = 0.f;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            if (j >= n) break;
-            const float gj = sh.ginv[r * NP + j];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) T[k] += gj * fmat[j * NP + k];
-        }
-        // GG = -T G^-1 (row r)
-        float GG[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) GG[k] = 0.f;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            if (j >= n) break;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) GG[k] -= T[j] * sh.ginv[j * NP + k];
-        }
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            const cpx<float> c = sh.myrow[k];
-            const float cm2 = norm2(c);
-            const cpx<float> ph = cm2 > 0.f ? rsqrtf(cm2) * c : mk<float>(0.f, 0.f);
-            h[k] = sh.ginv[r * NP + k] * h[k] + ((1.f - beta) * GG[k]) * ph;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < NP; ++k)
-        if (k == r || k >= n || !S.live) h[k] = mk<float>(0.f, 0.f);
-
-    // C -> S.
-    {
-        float P[NP];
-        float rowsum = 0.f;
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            const cpx<float> c = sh.myrow[k];
-            P[k] = h[k].x * c.x + h[k].y * c.y;
-            rowsum += P[k];
-        }
-        publish<NP, float>(P, fmat, r, gmask);
-        float colsum = 0.f;
-#pragma unroll
-        for (int i = 0; i < NP; ++i) colsum += fmat[i * NP + r];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) h[k] = (S.rsr * sh.rsg[k]) * h[k];
-        if (S.live && S.sr > 0.f) h[r] = mk<float>(-(rowsum + colsum) / (2.f * S.sr), 0.f);
-    }
-
-    // H = GS + GS^H (row r)
-    publish<NP, cpx<float>>(h, cmat, r, gmask);
-#pragma unroll
-    for (int k = 0; k < NP; ++k) h[k] = h[k] + conj(cmat[k * NP + r]);
-    __syncwarp(gmask);
-}
-
-// Coherence row r of pixel p, unit diagonal, into the lane's row cache.
-template <int NP>
-__device__ __forceinline__ void adj_load_row(cpx<float> *myrow, const float2 *__restrict__ Cpix, int r, int n) {
-    const bool live = r < n;
-    const int base_r = r * n - r * (r - 1) / 2 - r;
-    int idx_col = r;
-    cpx<float> v[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        v[k] = mk<float>((!live && k == r) ? 1.f : 0.f, 0.f);
-        if (live && k < n) {
-            if (k >= r) {
-                const float2 c = __ldg(Cpix + base_r + k);
-                v[k] = mk<float>(c.x, c.y);
-            } else {
-                const float2 c = __ldg(Cpix + idx_col);
-                v[k] = mk<float>(c.x, -c.y);
-                idx_col += n - k - 1;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < NP; ++k) myrow[k] = v[k];
-}
-
 // Per output pixel: H_p from the coherence C (packed), the diagonal sums and
-// the phase weights w [n][npx].  Pixels without data get H_p = 0.
+// the phase weights w [n][npx].  Pixels without data get H_p = 0.  With
+// K = GC + GC^H off the diagonal, H_rk = K_rk / sqrt(S_rr S_kk) and H_rr =
+// -sum_k Re(conj(K_rk) C_rk) / S_rr; K_rk = -g_rk (u_r conj(v_k) + v_r conj(u_k))
+// + (1 - beta) (GG_rk + GG_kr) C_rk / |C_rk|.
+// What bounds it is instruction issue and fetch: a pixel is two eliminations
+// and two products of N x N matrices by one warp.  The products used to be
+// unrolled over both indices, 576 to 1024 multiply-adds of straight-line code
+// each that every warp fetched for itself, in rows of 24 or 32 entries; as
+// loops over the rows, in rows of 20 to 32 entries in steps of 4, with G^-1
+// taken from the solve instead of inverted again, 301 x 403 pixels at stride 1
+// take 2.88 instead of 5.36 ms at N = 20, 7.6 instead of 12.4 ms at N = 28 and
+// 0.99 instead of 1.38 ms at N = 14.
+constexpr int kAdjWarps = 2;
+
 template <int NP>
-__global__ void __launch_bounds__(kAdjWarps * 32) k_adj_pixel(const float2 *__restrict__ C,
-                                                              const float *__restrict__ Sd, int n, long long npx,
-                                                              int ref, const EmiParams prm,
-                                                              const float *__restrict__ w,
-                                                              float2 *__restrict__ Hout) {
-    constexpr bool kPow2 = (NP & (NP - 1)) == 0;
-    constexpr int G = kPow2 ? 32 / NP : 1;
-    constexpr int kRowPitch = NP + 2;
-    constexpr int kGrpBuf = 2 * NP + 2;
-    __shared__ __align__(16) cpx<float> sbuf[kAdjWarps][G * kGrpBuf];
-    __shared__ __align__(16) cpx<float> rowcache[kAdjWarps * 32 * kRowPitch];
-    __shared__ __align__(16) cpx<float> mats[kAdjWarps][32 * NP];  // one NP x NP matrix per group
+struct AdjMinBlocks {
+    static constexpr int value = NP > 24 ? 5 : (NP > 16 ? 7 : 8);
+};
+
+template <int NP>
+__global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
+    k_adj_pixel(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref,
+                const EmiParams prm, const float *__restrict__ w, float2 *__restrict__ Hout) {
+    using Sh = AdjShared<NP>;
+    constexpr int G = Sh::G, P = Sh::kPitch;
+    constexpr int kBytes = Sh::oG + Sh::kMat;
+    __shared__ __align__(16) char smem[kAdjWarps * G * kBytes];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = kPow2 ? lane / NP : 0, r = lane - grp * NP;  // 24-entry rows: one pixel a warp
-    const int glane0 = grp * NP;
-    const unsigned gmask = (NP >= 24) ? 0xffffffffu : (((1u << NP) - 1u) << glane0);
+    const AdjLane<NP> L(lane);
+    const int r = L.r, rr = L.rr, grp = L.glane0 / NP;
+    const unsigned gmask = L.gmask;
+    const Sh sh{smem + (warp * G + grp) * kBytes};
     const long long nt = ntri(n);
     const long long step = (long long)gridDim.x * kAdjWarps * G;
-    cpx<float> *myrow = rowcache + (size_t)(warp * 32 + lane) * kRowPitch;
-    cpx<float> *cbuf = &sbuf[warp][grp * kGrpBuf];
-    float *rbuf = reinterpret_cast<float *>(cbuf);
-    cpx<float> *cmat = &mats[warp][grp * NP * NP];
-    float *fmat = reinterpret_cast<float *>(cmat);
     EmiParams q = prm;
     q.fp64_resolve = 0;  // the adjoint differentiates the single-precision solve
 
@@ -313,150 +263,124 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adj_pixel(const float2 *__re
                 for (int k = r; k < n; ++k) Hout[p * nt + packed_index(n, r, k)] = make_float2(0.f, 0.f);
             continue;
         }
+        adj_load<NP>(sh, Cpix, r, n);
+        __syncwarp(gmask);
+        AdjPixel<NP> S;
+        cpx<float> u;
         {
-            const int base_r = r * n - r * (r - 1) / 2 - r;
-            int idx_col = r;
-            cpx<float> v[NP];
+            cpx<float> mrow[NP];
+            adj_prepare<NP>(S, mrow, sh, L, Sd, p, n, ref, q);
+            // Gradient on v (gauge-free), projected orthogonal to v.
+            const float wr = live ? __ldg(w + (long long)r * npx + p) : 0.f;
+            const float wsum = group_sum<NP, float>(live && r != ref ? wr : 0.f, gmask);
+            const float m2 = norm2(S.v);
+            const float coef = (r == ref) ? -wsum : wr;
+            cpx<float> gv = (live && m2 > 0.f) ? (coef / m2) * mk<float>(-S.v.y, S.v.x) : mk<float>(0.f, 0.f);
+            const cpx<float> t = conj(S.v) * gv;
+            const float sx = group_sum<NP, float>(t.x, gmask), sy = group_sum<NP, float>(t.y, gmask);
+            gv = gv - S.v * mk<float>(sx, sy);
+            // u = M g_v  (orthogonal to v)
+            u = group_matvec<NP, float>(mrow, gv, sh.buf(), r, gmask);
+        }
+        cpx<float> *uall = sh.buf();
+        const cpx<float> *Crow = sh.C() + rr * P, *vg = sh.v();
+        const float *gcol = sh.g() + rr;
+        uall[r] = u;
+        float GG[NP];
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                v[k] = mk<float>((!live && k == r) ? 1.f : 0.f, 0.f);
-                if (live && k < n) {
-                    if (k >= r) {
-                        const float2 c = __ldg(Cpix + base_r + k);
-                        v[k] = mk<float>(c.x, c.y);
-                    } else {
-                        const float2 c = __ldg(Cpix + idx_col);
-                        v[k] = mk<float>(c.x, -c.y);
-                        idx_col += n - k - 1;
+        for (int k = 0; k < NP; ++k) GG[k] = 0.f;
+        if (!S.evd) {
+            // R = Re(conj(GA) o C), GA = -u v^H (row r); GG = -G^-1 R G^-1.  The
+            // products run over the rows of R and G^-1 in loops that are not
+            // unrolled over the row index (short code), the left factor's
+            // entry read from shared memory and the right factor's row as
+            // broadcast 16-byte loads.
+            float *R = sh.M(), *T = sh.M() + NP * NP;
+            if (r < NP) {
+                float rrow[NP];  // -R
+#pragma unroll
+                for (int k = 0; k < NP; k += 2) {
+                    cpx<float> c[2], v[2];
+                    load_pair(Crow + k, c);
+                    load_pair(vg + k, v);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const cpx<float> t = c[e] * v[e];
+                        rrow[k + e] = u.x * t.x + u.y * t.y;
                     }
                 }
+                store_row<NP>(R + rr * NP, rrow);
             }
+            __syncwarp(gmask);
+#pragma unroll 2
+            for (int j = 0; j < n; ++j) {
+                const float gj = gcol[j * NP];
+                const float4 *row = reinterpret_cast<const float4 *>(R + j * NP);
 #pragma unroll
-            for (int k = 0; k < NP; ++k) myrow[k] = v[k];
-        }
-        __syncwarp(gmask);
-        const AdjRow<NP> ld{myrow};
-        const PixelResult res = emi_solve<NP, float>(ld, r, n, ref, q, cbuf, gmask, glane0, false);
-        const cpx<float> v = live ? res.v : mk<float>(0.f, 0.f);
-
-        // Gradient on v (gauge-free), projected orthogonal to v.
-        const float wr = live ? __ldg(w + (long long)r * npx + p) : 0.f;
-        const float wsum = group_sum<NP, float>(live && r != ref ? wr : 0.f, gmask);
-        const float m2 = norm2(v);
-        const float coef = (r == ref) ? -wsum : wr;
-        cpx<float> gv = (live && m2 > 0.f) ? (coef / m2) * mk<float>(-v.y, v.x) : mk<float>(0.f, 0.f);
-        {
-            const cpx<float> t = conj(v) * gv;
-            const float sx = group_sum<NP, float>(t.x, gmask), sy = group_sum<NP, float>(t.y, gmask);
-            gv = gv - v * mk<float>(sx, sy);
-        }
-
-        // A row (C, or G^-1 o C) and G^-1 row.
-        cpx<float> crow[NP], a[NP];
-        float gi[NP];
-        load_crow<NP, float>(crow, ld, r, n);
+                for (int q4 = 0; q4 < NP / 4; ++q4) {
+                    const float4 x = row[q4];
+                    GG[q4 * 4 + 0] += gj * x.x;
+                    GG[q4 * 4 + 1] += gj * x.y;
+                    GG[q4 * 4 + 2] += gj * x.z;
+                    GG[q4 * 4 + 3] += gj * x.w;
+                }
+            }
+            if (r < NP) {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            float m = mag_t(norm2(crow[k]));
-            if (q.beta != 0.f) m = (1.f - q.beta) * m + ((k == r) ? q.beta : 0.f);
-            gi[k] = m;
-        }
-        if (!res.evd) gj_invert<NP, float, float, true>(gi, rbuf, r, n, gmask, 0.f);
-#pragma unroll
-        for (int k = 0; k < NP; ++k) a[k] = res.evd ? crow[k] : mk<float>(gi[k] * crow[k].x, gi[k] * crow[k].y);
-        // lambda = v^H A v (the eigenvalue the perturbation is about)
-        const cpx<float> av = group_matvec<NP, float>(a, v, cbuf, r, gmask);
-        const float lam = group_sum<NP, float>(live ? (v.x * av.x + v.y * av.y) : 0.f, gmask);
-        // every lane's v
-        cpx<float> vv[NP];
-        cbuf[r] = v;
-        __syncwarp(gmask);
-#pragma unroll
-        for (int k = 0; k < NP; ++k) vv[k] = cbuf[k];
-        __syncwarp(gmask);
-        // u = (A - lambda I + c v v^H)^-1 g_v  (c keeps the deflated matrix well scaled)
-        const float cdef = fmaxf(1.f, fabsf(lam));
-        cpx<float> mrow[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            mrow[k] = a[k] + cdef * (v * conj(vv[k]));
-            if (k == r && live) mrow[k].x -= lam;
-        }
-        gj_invert<NP, float, cpx<float>, false>(mrow, cbuf, r, n, gmask, 0.f);
-        const cpx<float> u = group_matvec<NP, float>(mrow, gv, cbuf, r, gmask);
-
-        // GA = -u v^H (row r), then GC (off the diagonal).
-        cpx<float> gc[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) gc[k] = mk<float>(0.f, 0.f) - u * conj(vv[k]);  // GA for now
-        if (!res.evd) {
-            float R[NP];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) R[k] = gc[k].x * crow[k].x + gc[k].y * crow[k].y;  // Re(conj(GA) C)
-            // T = G^-1 R (row r): sum_j gi[j] R_j.
-            publish<NP, float>(R, fmat, r, gmask);
-            float T[NP];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) T[k] = 0.f;
-#pragma unroll
-            for (int j = 0; j < NP; ++j)
-#pragma unroll
-                for (int k = 0; k < NP; ++k) T[k] += gi[j] * fmat[j * NP + k];
-            // GG = -T G^-1 (row r): -sum_j T[j] Ginv_j.
-            publish<NP, float>(gi, fmat, r, gmask);
-            float GG[NP];
+                for (int k = 0; k < NP; ++k) T[k * NP + rr] = GG[k];
+            }
 #pragma unroll
             for (int k = 0; k < NP; ++k) GG[k] = 0.f;
+#pragma unroll 2
+            for (int j = 0; j < n; ++j) {
+                const float tj = T[j * NP + rr];
+                const float4 *row = reinterpret_cast<const float4 *>(sh.g() + j * NP);
 #pragma unroll
-            for (int j = 0; j < NP; ++j)
+                for (int q4 = 0; q4 < NP / 4; ++q4) {
+                    const float4 x = row[q4];
+                    GG[q4 * 4 + 0] += tj * x.x;
+                    GG[q4 * 4 + 1] += tj * x.y;
+                    GG[q4 * 4 + 2] += tj * x.z;
+                    GG[q4 * 4 + 3] += tj * x.w;
+                }
+            }
+            // GG + GG^T: the transpose through R (every lane is past its reads of it)
+            __syncwarp(gmask);
+            if (r < NP) store_row<NP>(R + rr * NP, GG);
+            __syncwarp(gmask);
 #pragma unroll
-                for (int k = 0; k < NP; ++k) GG[k] -= T[j] * fmat[j * NP + k];
+            for (int k = 0; k < NP; ++k) GG[k] = (1.f - q.beta) * (GG[k] + R[k * NP + rr]);
+        }
+        __syncwarp(gmask);
+        // Row r of K, its diagonal, and H, written as the columns of the packed
+        // upper triangle's rows: lane k writes H_ik = conj(H_ki) for i <= k, a
+        // run of consecutive addresses across the lanes.
+        cpx<float> h[NP];
+        float diag = 0.f;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const float cm2 = norm2(crow[k]);
-                const cpx<float> ph = cm2 > 0.f ? rsqrtf(cm2) * crow[k] : mk<float>(0.f, 0.f);
-                gc[k] = gi[k] * gc[k] + ((1.f - q.beta) * GG[k]) * ph;
+        for (int k2 = 0; k2 < NP; k2 += 2) {
+            cpx<float> cc[2], vv[2], uu[2];
+            load_pair(Crow + k2, cc);
+            load_pair(vg + k2, vv);
+            load_pair(uall + k2, uu);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int k = k2 + e;
+                const cpx<float> c = cc[e], t = u * conj(vv[e]) + S.v * conj(uu[e]);
+                const float m2 = norm2(c), g = gcol[k * NP];
+                const float a = m2 > 0.f ? rsqrtf(m2) * GG[k] : 0.f;
+                h[k] = k == r ? mk<float>(0.f, 0.f) : mk<float>(a * c.x - g * t.x, a * c.y - g * t.y);
+                diag += h[k].x * c.x + h[k].y * c.y;
             }
         }
-#pragma unroll
-        for (int k = 0; k < NP; ++k)
-            if (k == r || k >= n || !live) gc[k] = mk<float>(0.f, 0.f);
-
-        // C -> S.
-        const float sr = live ? __ldg(Sd + p * n + r) : 0.f;
-        const float rsr = sr > 0.f ? rsqrtf(sr) : 0.f;
-        float rs[NP];
-        rbuf[r] = rsr;
-        __syncwarp(gmask);
-#pragma unroll
-        for (int k = 0; k < NP; ++k) rs[k] = rbuf[k];
-        __syncwarp(gmask);
-        float P[NP];
-        float rowsum = 0.f;
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            P[k] = gc[k].x * crow[k].x + gc[k].y * crow[k].y;
-            rowsum += P[k];
-        }
-        publish<NP, float>(P, fmat, r, gmask);
-        float colsum = 0.f;
-#pragma unroll
-        for (int i = 0; i < NP; ++i) colsum += fmat[i * NP + r];
-        cpx<float> gs[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) gs[k] = (rsr * rs[k]) * gc[k];
-        if (live && sr > 0.f) gs[r] = mk<float>(-(rowsum + colsum) / (2.f * sr), 0.f);
-
-        // H = GS + GS^H, packed upper triangle.
-        publish<NP, cpx<float>>(gs, cmat, r, gmask);
         if (live) {
             float2 *Hp = Hout + p * nt;
 #pragma unroll
-            for (int k = 0; k < NP; ++k)
-                if (k >= r && k < n) {
-                    const cpx<float> h = gs[k] + conj(cmat[k * NP + r]);
-                    Hp[packed_index(n, r, k)] = make_float2(h.x, h.y);
-                }
+            for (int k = 0; k < NP; ++k) {
+                const float s = S.rsr * sh.rs()[k];
+                if (k < r) Hp[packed_index(n, k, r)] = make_float2(s * h[k].x, -s * h[k].y);
+                if (k == r) Hp[packed_index(n, k, r)] = make_float2(-S.rsr * S.rsr * diag, 0.f);
+            }
         }
         __syncwarp(gmask);
     }
@@ -466,95 +390,264 @@ __global__ void __launch_bounds__(kAdjWarps * 32) k_adj_pixel(const float2 *__re
 // every SLC sample, E|n|^2 = sigma2, propagated through the linked phases.
 // With g(q) = H_p z(q) the gradient of phihat_i(p) over the pixel's masked
 // window, Var phihat_i = (sigma2 / 2) sum_q |g(q)|^2 = (sigma2 / 2) tr(H^H H S),
-// S = sum_q m(q) z(q) z(q)^H, S_jk = C_jk sqrt(S_jj S_kk).  H is Hermitian, so
-// tr(H^H H S) = sum_k <row k of H, row k of H S>: each lane's own rows.
-// One pass per date with the weight e_i; the reference date has 0.  One warp
-// a CTA (the shared buffers of a 32-lane group take 30 KB).
-constexpr int kUncWarps = 1;
+// S = sum_q m(q) z(q) z(q)^H = D C D, D = diag(sqrt(S_kk)), and H = D^-1 K D^-1
+// (K as in k_adj_pixel, K_rr = -sum_k Re(conj(K_rk) C_rk)), so
+//     Var phihat_i = (sigma2 / 2) sum_r (1 / S_rr) k_r C k_r^H,   k_r row r of K.
+// What depends on the date i is u^(i) = M_:i c_i - M_:ref c_ref, c = j v / |v|^2
+// (columns of M: the weight e_i needs no product), so the pixel is prepared
+// once and every date costs
+//   GG = G^-1 [diag(Re u) X + diag(Im u) Y],  X + jY = (C diag(v)) G^-1
+// (X, Y formed once: 2 N^2 products a row and no intermediate matrix), the row
+// k_r, and its quadratic form over one triangle of C (Hermitian: half the
+// products of k_r C).
+// W warps share a prepared pixel (G pixels) and take two dates a pass; a pass
+// reads each row of X, Y and C once for both, as broadcast 16-byte loads in
+// loops that are not unrolled over the row index (short code).
+// One product H S and two with G^-1 for every date, unrolled, took 17.5 ms on
+// 201 x 301 pixels at stride 1 and N = 20, this 7.7 ms; 101 x 301 pixels at N =
+// 28 38.9 and 9.0 ms, 201 x 301 at N = 12 2.42 and 1.79 ms.
+template <int NP>
+struct UncCfg {
+    static constexpr int W = 2;
+    using Sh = AdjShared<NP>;
+    static constexpr int oU = Sh::oG + Sh::kMat;       // u [date][r]
+    static constexpr int oK = oU + 2 * Sh::kMat;       // per warp, two dates: rows k_r [NP][NP + 1]
+    static constexpr int kKPitch = NP + 1;             // odd: a lane reads its own row 8 bytes at a time
+    static constexpr int kK = NP * kKPitch * 8;        // one date's rows
+    static constexpr int kBytes = oK + W * 2 * kK;     // of one group
+    static_assert(NP * (NP + 1) * 4 <= kK, "the transposed products fit the row buffers");
+    static constexpr int kSmem = Sh::G * kBytes;
+    // register budget: what shared memory lets an SM hold
+    static constexpr int kMinBlocks = NP > 28 ? 3 : (NP > 24 ? 4 : (NP > 20 ? 5 : 7));
+};
 
 template <int NP>
-__global__ void __launch_bounds__(kUncWarps * 32) k_adj_uncert(const float2 *__restrict__ C,
-                                                               const float *__restrict__ Sd, int n, long long npx,
-                                                               int ref, const EmiParams prm, float sigma2,
-                                                               float *__restrict__ sd_out) {
-    constexpr bool kPow2 = (NP & (NP - 1)) == 0;
-    constexpr int G = kPow2 ? 32 / NP : 1;
-    constexpr int kRowPitch = NP + 2;
-    constexpr int kGrpBuf = 2 * NP + 2;
-    __shared__ __align__(16) cpx<float> sbuf[kUncWarps][G * kGrpBuf];
-    __shared__ __align__(16) cpx<float> rowcache[kUncWarps * 32 * kRowPitch];
-    __shared__ __align__(16) cpx<float> mats[kUncWarps][32 * NP];
-    __shared__ __align__(16) cpx<float> smats[kUncWarps][32 * NP];  // S of the group's pixel
-    __shared__ __align__(16) float ginvs[kUncWarps][32 * NP];       // G^-1 of the group's pixel
-    __shared__ __align__(16) cpx<float> vs[kUncWarps][32];
-    __shared__ __align__(16) float rss[kUncWarps][32];
+__global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
+    k_adj_uncert(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref, const EmiParams prm,
+                 float sigma2, float *__restrict__ sd_out) {
+    using Cfg = UncCfg<NP>;
+    using Sh = AdjShared<NP>;
+    constexpr int G = Sh::G, P = Sh::kPitch, W = Cfg::W;
+    extern __shared__ __align__(16) char unc_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = kPow2 ? lane / NP : 0, r = lane - grp * NP;  // 24-entry rows: one pixel a warp
-    const int glane0 = grp * NP;
-    const unsigned gmask = (NP >= 24) ? 0xffffffffu : (((1u << NP) - 1u) << glane0);
+    const AdjLane<NP> L(lane);
+    const int r = L.r, rr = L.rr, grp = L.glane0 / NP;
+    const unsigned gmask = L.gmask;
+    char *gbase = unc_smem + grp * Cfg::kBytes;
+    const Sh sh{gbase};
+    cpx<float> *U = reinterpret_cast<cpx<float> *>(gbase + Cfg::oU);
+    cpx<float> *K[2];
+    float *Pt[2];
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        K[d] = reinterpret_cast<cpx<float> *>(gbase + Cfg::oK + (warp * 2 + d) * Cfg::kK);
+        Pt[d] = reinterpret_cast<float *>(K[d]);
+    }
+    float2 *XY = reinterpret_cast<float2 *>(sh.M());
+    const cpx<float> *Crow = sh.C() + rr * P, *vg = sh.v();
+    const float *gcol = sh.g() + rr;
     const long long nt = ntri(n);
-    const long long step = (long long)gridDim.x * kUncWarps * G;
-    cpx<float> *myrow = rowcache + (size_t)(warp * 32 + lane) * kRowPitch;
-    cpx<float> *cbuf = &sbuf[warp][grp * kGrpBuf];
-    cpx<float> *cmat = &mats[warp][grp * NP * NP];
-    cpx<float> *smat = &smats[warp][grp * NP * NP];
-    const UncShared<NP> sh{myrow, &vs[warp][glane0], &rss[warp][glane0], &ginvs[warp][grp * NP * NP]};
+    const long long step = (long long)gridDim.x * G;
     EmiParams q = prm;
     q.fp64_resolve = 0;
     const float qnan = __int_as_float(0x7fc00000);
+    const bool live = r < n;
+    __shared__ int s_evd[G];
 
-    for (long long base = ((long long)blockIdx.x * kUncWarps + warp) * G; base < npx; base += step) {
+    for (long long base = (long long)blockIdx.x * G; base < npx; base += step) {
         const long long p = base + grp;
         const bool valid = p < npx;
         const float2 *Cpix = C + (valid ? p : 0) * nt;
-        const bool live = r < n;
         bool nan = false;
         if (valid && live) nan = isnan(__ldg(Cpix + packed_index(n, r, r)).x);
         nan = __any_sync(gmask, nan);
-        if (!valid) continue;
-        if (nan) {
-            if (live) sd_out[(long long)r * npx + p] = qnan;
-            continue;
-        }
-        adj_load_row<NP>(myrow, Cpix, r, n);
-        __syncwarp(gmask);
-        AdjPixelState<NP> S;
-        adj_prepare<NP>(S, sh, Sd, p, r, n, ref, q, cbuf, gmask, glane0);
-        // S rows (unnormalised): S_rk = C_rk sqrt(S_rr S_kk)
-        {
-            // sqrt(S_rr S_kk) = sqrt(S_rr) / rs_k, rs_k = 1 / sqrt(S_kk) (0 where S_kk = 0)
-            const float sq_r = sqrtf(S.sr);
-            cpx<float> srow[NP];
+        const bool solve = valid && !nan;
+        if (warp == 0 && valid) {
+            if (live && (nan || r == ref)) sd_out[(long long)r * npx + p] = nan ? qnan : 0.f;
+            if (solve) {
+                adj_load<NP>(sh, Cpix, r, n);
+                __syncwarp(gmask);
+                AdjPixel<NP> S;
+                {
+                    cpx<float> mrow[NP];
+                    adj_prepare<NP>(S, mrow, sh, L, Sd, p, n, ref, q);
+                    if (r == 0) s_evd[grp] = S.evd;
+                    // u of every date; g_v has no component along v except where
+                    // v_i or v_ref is exactly 0 (M v = v / c)
+                    const cpx<float> cv = (1.f / S.cdef) * mk<float>(-S.v.y, S.v.x);
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const float rk = sh.rsg[k];
-                srow[k] = (live && k < n && rk > 0.f) ? (sq_r / rk) * myrow[k] : mk<float>(0.f, 0.f);
-            }
-            publish<NP, cpx<float>>(srow, smat, r, gmask);
-        }
-        float sd_mine = 0.f;  // this lane's date
-        for (int i = 0; i < n; ++i) {
-            if (i == ref) continue;  // uniform across the group
-            cpx<float> h[NP];
-            adj_h_row<NP>(S, sh, (r == i) ? 1.f : 0.f, r, n, ref, q.beta, cbuf, cmat, gmask, h);
-            // row r of M = H S, then <row r of H, row r of M>
-            float tr = 0.f;
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                if (k >= n) break;  // S and H are zero past n
-                cpx<float> m = mk<float>(0.f, 0.f);
-#pragma unroll
-                for (int j = 0; j < NP; ++j) {
-                    if (j >= n) break;
-                    m = cfma(h[j], smat[j * NP + k], m);
+                    for (int i = 0; i < NP; ++i) {
+                        const cpx<float> vi = vg[i];
+                        const float m2 = norm2(vi);
+                        const cpx<float> ci = m2 > 0.f ? (1.f / m2) * mk<float>(-vi.y, vi.x) : mk<float>(0.f, 0.f);
+                        cpx<float> ui = mrow[i] * ci;
+                        if (m2 > 0.f) ui = ui - cv;
+                        if (r < NP) U[i * NP + r] = ui;
+                    }
                 }
-                tr += h[k].x * m.x + h[k].y * m.y;  // Re(conj(h_k) m_k)
+                const cpx<float> uref = U[ref * NP + rr];
+#pragma unroll 4
+                for (int i = 0; i < n; ++i)
+                    if (r < NP) U[i * NP + r] = U[i * NP + r] - uref;
+                // X + jY over the row slots of the solve (read by now: M's inversion syncs)
+                float X[NP], Y[NP];
+#pragma unroll
+                for (int k = 0; k < NP; ++k) X[k] = Y[k] = 0.f;
+#pragma unroll 1
+                for (int m = 0; m < n; ++m) {
+                    const cpx<float> t = vg[m] * Crow[m];
+                    const float4 *row = reinterpret_cast<const float4 *>(sh.g() + m * NP);
+#pragma unroll
+                    for (int q4 = 0; q4 < NP / 4; ++q4) {
+                        const float4 g4 = row[q4];
+                        X[q4 * 4 + 0] += t.x * g4.x;
+                        Y[q4 * 4 + 0] += t.y * g4.x;
+                        X[q4 * 4 + 1] += t.x * g4.y;
+                        Y[q4 * 4 + 1] += t.y * g4.y;
+                        X[q4 * 4 + 2] += t.x * g4.z;
+                        Y[q4 * 4 + 2] += t.y * g4.z;
+                        X[q4 * 4 + 3] += t.x * g4.w;
+                        Y[q4 * 4 + 3] += t.y * g4.w;
+                    }
+                }
+                if (r < NP) {
+                    float4 *dst = reinterpret_cast<float4 *>(XY + r * NP);
+#pragma unroll
+                    for (int k = 0; k < NP; k += 2) dst[k / 2] = make_float4(X[k], Y[k], X[k + 1], Y[k + 1]);
+                }
             }
-            tr = group_sum<NP, float>(live ? tr : 0.f, gmask);
-            if (r == i) sd_mine = sqrtf(fmaxf(0.5f * sigma2 * tr, 0.f));
         }
-        if (live) sd_out[(long long)r * npx + p] = sd_mine;  // 0 at the reference date
-        __syncwarp(gmask);
+        __syncthreads();
+        if (solve) {
+            const bool evd = s_evd[grp] != 0;
+            const float rsr = sh.rs()[r];
+            const cpx<float> vr = vg[r];
+            for (int i0 = 2 * warp; i0 < n; i0 += 2 * W) {
+                const int i1 = i0 + 1 < n ? i0 + 1 : i0;
+                const cpx<float> *U0 = U + i0 * NP, *U1 = U + i1 * NP;
+                float A0[NP], A1[NP];
+#pragma unroll
+                for (int k = 0; k < NP; ++k) A0[k] = A1[k] = 0.f;
+                if (!evd) {
+#pragma unroll 1
+                    for (int j = 0; j < n; ++j) {
+                        const float g = gcol[j * NP];
+                        const cpx<float> u0 = g * U0[j], u1 = g * U1[j];
+                        const float4 *row = reinterpret_cast<const float4 *>(XY + j * NP);
+#pragma unroll
+                        for (int k = 0; k < NP; k += 2) {
+                            const float4 t = row[k / 2];
+                            A0[k] += u0.x * t.x;
+                            A0[k] += u0.y * t.y;
+                            A0[k + 1] += u0.x * t.z;
+                            A0[k + 1] += u0.y * t.w;
+                            A1[k] += u1.x * t.x;
+                            A1[k] += u1.y * t.y;
+                            A1[k + 1] += u1.x * t.z;
+                            A1[k + 1] += u1.y * t.w;
+                        }
+                    }
+                    // GG + GG^T through the row buffers
+                    if (r < NP) {
+#pragma unroll
+                        for (int k = 0; k < NP; ++k) {
+                            Pt[0][k * (NP + 1) + r] = A0[k];
+                            Pt[1][k * (NP + 1) + r] = A1[k];
+                        }
+                    }
+                    __syncwarp(gmask);
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) {
+                        A0[k] += Pt[0][rr * (NP + 1) + k];
+                        A1[k] += Pt[1][rr * (NP + 1) + k];
+                    }
+                    __syncwarp(gmask);
+                }
+                // Rows k_r of both dates into this lane's row buffers.
+                const cpx<float> ur0 = U0[rr], ur1 = U1[rr];
+                float diag0 = 0.f, diag1 = 0.f;
+                cpx<float> *k0 = K[0] + rr * Cfg::kKPitch, *k1 = K[1] + rr * Cfg::kKPitch;
+#pragma unroll
+                for (int k2 = 0; k2 < NP; k2 += 2) {
+                    cpx<float> cc[2], vv[2], w0[2], w1[2];
+                    load_pair(Crow + k2, cc);
+                    load_pair(vg + k2, vv);
+                    load_pair(U0 + k2, w0);
+                    load_pair(U1 + k2, w1);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int k = k2 + e;
+                        const cpx<float> c = cc[e];
+                        const float m2 = norm2(c), g = gcol[k * NP];
+                        const float im = m2 > 0.f ? (1.f - q.beta) * rsqrtf(m2) : 0.f;
+                        const cpx<float> t0 = ur0 * conj(vv[e]) + vr * conj(w0[e]);
+                        const cpx<float> t1 = ur1 * conj(vv[e]) + vr * conj(w1[e]);
+                        const float a0 = im * A0[k], a1 = im * A1[k];
+                        cpx<float> h0 = mk<float>(a0 * c.x - g * t0.x, a0 * c.y - g * t0.y);
+                        cpx<float> h1 = mk<float>(a1 * c.x - g * t1.x, a1 * c.y - g * t1.y);
+                        if (k == r) h0 = h1 = mk<float>(0.f, 0.f);
+                        diag0 += h0.x * c.x + h0.y * c.y;
+                        diag1 += h1.x * c.x + h1.y * c.y;
+                        if (r < NP) {
+                            k0[k] = h0;
+                            k1[k] = h1;
+                        }
+                    }
+                }
+                if (r < NP) {
+                    k0[r] = mk<float>(-diag0, 0.f);
+                    k1[r] = mk<float>(-diag1, 0.f);
+                }
+                // k C k^H = Re sum_m conj(k_m) sum_l w_lm k_l C_lm over blocks of
+                // columns m: weight 1 inside the diagonal block (both orders
+                // of a pair appear), 2 below it (one order).
+                float q0 = 0.f, q1 = 0.f;
+#pragma unroll
+                for (int mb = 0; mb < NP; mb += 8) {
+                    constexpr int kB = 8;
+                    const int width = NP - mb < kB ? NP - mb : kB;
+                    if (mb >= n) break;
+                    cpx<float> s0[kB], s1[kB];
+#pragma unroll
+                    for (int e = 0; e < kB; ++e) s0[e] = s1[e] = mk<float>(0.f, 0.f);
+#pragma unroll 1
+                    for (int l = mb; l < n; ++l) {
+                        const float wl = l < mb + kB ? 1.f : 2.f;
+                        const cpx<float> a0 = wl * k0[l], a1 = wl * k1[l];
+                        const float4 *row = reinterpret_cast<const float4 *>(sh.C() + l * P + mb);
+#pragma unroll
+                        for (int e = 0; e < kB; e += 2) {
+                            if (e < width) {
+                                const float4 t = row[e / 2];
+                                const cpx<float> ca = mk<float>(t.x, t.y), cb = mk<float>(t.z, t.w);
+                                s0[e] = cfma(a0, ca, s0[e]);
+                                s0[e + 1] = cfma(a0, cb, s0[e + 1]);
+                                s1[e] = cfma(a1, ca, s1[e]);
+                                s1[e + 1] = cfma(a1, cb, s1[e + 1]);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < kB; ++e) {
+                        if (e < width) {
+                            const cpx<float> a0 = k0[mb + e], a1 = k1[mb + e];
+                            q0 += a0.x * s0[e].x + a0.y * s0[e].y;
+                            q1 += a1.x * s1[e].x + a1.y * s1[e].y;
+                        }
+                    }
+                }
+                const float s2 = live ? rsr * rsr : 0.f;
+                const float tr0 = group_sum<NP, float>(s2 > 0.f ? s2 * q0 : 0.f, gmask);
+                const float tr1 = group_sum<NP, float>(s2 > 0.f ? s2 * q1 : 0.f, gmask);
+                if (r == 0) {
+                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = sqrtf(fmaxf(0.5f * sigma2 * tr0, 0.f));
+                    if (i1 != i0 && i1 != ref)
+                        sd_out[(long long)i1 * npx + p] = sqrtf(fmaxf(0.5f * sigma2 * tr1, 0.f));
+                }
+                __syncwarp(gmask);  // the row buffers are free for the next pass
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -787,12 +880,27 @@ static cudaError_t run_adj_pixel(const float2 *C, const float *Sd, int n, long l
 template <int NP>
 static cudaError_t run_adj_uncert(const float2 *C, const float *Sd, int n, long long npx, int ref,
                                   const EmiParams &prm, float sigma2, float *out, cudaStream_t s) {
-    constexpr int G = (NP & (NP - 1)) ? 1 : 32 / NP;
-    long long blocks = ((npx + G - 1) / G + kUncWarps - 1) / kUncWarps;
+    using Cfg = UncCfg<NP>;
+    constexpr int G = AdjShared<NP>::G;
+    cudaError_t e = cudaFuncSetAttribute(k_adj_uncert<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+    if (e != cudaSuccess) return e;
     const long long cap = (long long)device_sm_count() * 32;
-    blocks = std::max<long long>(1, std::min(blocks, cap));
-    k_adj_uncert<NP><<<(unsigned)blocks, kUncWarps * 32, 0, s>>>(C, Sd, n, npx, ref, prm, sigma2, out);
+    const long long blocks = std::max<long long>(1, std::min((npx + G - 1) / G, cap));
+    k_adj_uncert<NP><<<(unsigned)blocks, Cfg::W * 32, Cfg::kSmem, s>>>(C, Sd, n, npx, ref, prm, sigma2, out);
     return cudaGetLastError();
+}
+
+// f(row length) for the rows of n dates (emi_row_length).
+template <class F>
+static cudaError_t with_row_length(int n, const F &f) {
+    switch (emi_row_length(n)) {
+        case 8: return f(std::integral_constant<int, 8>());
+        case 16: return f(std::integral_constant<int, 16>());
+        case 20: return f(std::integral_constant<int, 20>());
+        case 24: return f(std::integral_constant<int, 24>());
+        case 28: return f(std::integral_constant<int, 28>());
+        default: return f(std::integral_constant<int, 32>());
+    }
 }
 
 // Workspace layout: C [npx][ntri], H [npx][ntri], Sd [npx][n] (256-byte aligned parts).
@@ -821,10 +929,8 @@ static cudaError_t adjoint_h(const Planes &z, int n, const Geom &g, const uint64
     if (prof) prof->begin("adjoint_pixel", s);
     k_adj_sdiag<<<adj_grid(npx * n), 256, 0, s>>>(z, n, g, mask, Sd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (n <= 8) e = run_adj_pixel<8>(C, Sd, n, npx, ref, prm, dphase, H, s);
-    else if (n <= 16) e = run_adj_pixel<16>(C, Sd, n, npx, ref, prm, dphase, H, s);
-    else if (n <= 24) e = run_adj_pixel<24>(C, Sd, n, npx, ref, prm, dphase, H, s);
-    else e = run_adj_pixel<32>(C, Sd, n, npx, ref, prm, dphase, H, s);
+    e = with_row_length(
+        n, [&](auto np) { return run_adj_pixel<decltype(np)::value>(C, Sd, n, npx, ref, prm, dphase, H, s); });
     if (prof) prof->end(s);
     return e;
 }
@@ -902,10 +1008,8 @@ cudaError_t launch_phase_uncertainty(const Planes &z, int n, const Geom &g, cons
     if (e != cudaSuccess) return e;
     k_adj_sdiag<<<adj_grid(npx * n), 256, 0, s>>>(z, n, g, mask, Sd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (n <= 8) return run_adj_uncert<8>(C, Sd, n, npx, ref, prm, sigma2, sd, s);
-    if (n <= 16) return run_adj_uncert<16>(C, Sd, n, npx, ref, prm, sigma2, sd, s);
-    if (n <= 24) return run_adj_uncert<24>(C, Sd, n, npx, ref, prm, sigma2, sd, s);
-    return run_adj_uncert<32>(C, Sd, n, npx, ref, prm, sigma2, sd, s);
+    return with_row_length(
+        n, [&](auto np) { return run_adj_uncert<decltype(np)::value>(C, Sd, n, npx, ref, prm, sigma2, sd, s); });
 }
 
 }  // namespace plk
