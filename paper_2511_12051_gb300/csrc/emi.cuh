@@ -62,17 +62,28 @@ __device__ __forceinline__ T group_sum(T v, unsigned gmask) {
     for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(gmask, v, off);
     return v;
 }
+// Largest and smallest of non-negative values (0 for NaN): in single precision
+// one reduction of the bit patterns, which order as the values do, instead of
+// four or five exchanges (a 15-date solve 2% faster).
 template <int NP, class T>
 __device__ __forceinline__ T group_max(T v, unsigned gmask) {
+    if constexpr (sizeof(T) == 4) {
+        return __uint_as_float(__reduce_max_sync(gmask, __float_as_uint(fmax(v, T(0)))));
+    } else {
 #pragma unroll
-    for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmax(v, __shfl_xor_sync(gmask, v, off));
-    return v;
+        for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmax(v, __shfl_xor_sync(gmask, v, off));
+        return v;
+    }
 }
 template <int NP, class T>
 __device__ __forceinline__ T group_min(T v, unsigned gmask) {
+    if constexpr (sizeof(T) == 4) {
+        return __uint_as_float(__reduce_min_sync(gmask, __float_as_uint(fmax(v, T(0)))));
+    } else {
 #pragma unroll
-    for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmin(v, __shfl_xor_sync(gmask, v, off));
-    return v;
+        for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmin(v, __shfl_xor_sync(gmask, v, off));
+        return v;
+    }
 }
 
 // ---- scalar helpers over real T and complex cpx<T> -----------------------
@@ -149,10 +160,10 @@ __device__ __forceinline__ cpx<T> real_s(cpx<T>, T v) { return mk<T>(v, T(0)); }
 // whose inverse serves as a preconditioner); G has pivots <= 1.
 // PD = true (real G): a pivot <= tiny is replaced by tiny.  PD = false
 // (complex B, possibly indefinite): only a pivot of magnitude below tiny is.
-// Every lane sees every pivot, so all return the same value: the first real
-// pivot (in step order, over the first n steps, before replacement) that is
-// <= thr -- the one a Cholesky factorisation would stop at -- or, if there is
-// none, the smallest pivot.
+// Every lane sees every pivot, so all return the same value, over the n pivots
+// before replacement.  PD = true: the first pivot in step order that is <= thr
+// -- the one a Cholesky factorisation would stop at -- or, if there is none,
+// the smallest.  PD = false: the smallest pivot (thr unused).
 // a[c] <- a[(c + s) mod NP] for a group-uniform 0 <= s < NP.  Rows of 8 and
 // 16 entries: one conditional rotation per bit of s (NP moves each) instead of
 // s single-place shifts.  Rows beyond 16 entries (one pixel a warp, few padded
@@ -187,7 +198,9 @@ __device__ __forceinline__ void rotate_left(S (&a)[NP], int s) {
     }
 }
 
-template <int NP, class T, class S, bool PD>
+// ROT = false leaves the rows as the n steps leave them, a[c] holding column
+// (c + n) mod NP, for a consumer that multiplies them (rotated_slot).
+template <int NP, class T, class S, bool PD, bool ROT = true>
 __device__ __forceinline__ T gj_invert(S (&a)[NP], S *buf, int r, int n, unsigned gmask, T thr) {
     constexpr int E = 16 / sizeof(S);
     static_assert(NP % E == 0, "row must be a multiple of 16 bytes");
@@ -216,7 +229,7 @@ __device__ __forceinline__ T gj_invert(S (&a)[NP], S *buf, int r, int n, unsigne
             pr = re_s(p0[0]);
         }
         minpiv = fmin(minpiv, pr);
-        if (!have_low && pr <= thr) {
+        if (PD && !have_low && pr <= thr) {
             have_low = true;
             first_low = pr;
         }
@@ -247,11 +260,21 @@ __device__ __forceinline__ T gj_invert(S (&a)[NP], S *buf, int r, int n, unsigne
     // Padded pivots k >= n (identity row and column): f' = 0 on every lane and
     // the entry rotated in is the one rotated out, so each such step is a
     // rotation by one place; all of them together, a rotation by NP - n.
-    rotate_left<NP, S>(a, NP - n);
+    if constexpr (ROT) rotate_left<NP, S>(a, NP - n);
     return have_low ? first_low : minpiv;
 }
 
-// y = sum_j a[j] * v_j where v (one entry per lane) is published in buf.
+// Buffer slot of this lane's entry of a vector that multiplies rows left as
+// gj_invert<ROT = false> leaves them: column r stands at place (r - n) mod NP.
+// Publishing the vector rotated costs nothing; rotating the rows, two moves an
+// entry and padded pivot (rows beyond 16 entries: 40 to 56 moves for each).
+template <int NP>
+__device__ __forceinline__ int rotated_slot(int r, int n) {
+    return r >= NP ? r : (r >= n ? r - n : r - n + NP);
+}
+
+// y = sum_j a[j] * v_j where v (one entry per lane) is published in buf, this
+// lane's entry at place r.
 template <int NP, class T>
 __device__ __forceinline__ cpx<T> group_matvec(const cpx<T> (&a)[NP], cpx<T> v, cpx<T> *buf, int r,
                                                unsigned gmask) {
@@ -311,7 +334,45 @@ __device__ __forceinline__ void load_crow(cpx<T> (&c)[NP], const Loader &load, i
     }
 }
 
-// a <- (G^{-1} o C - mu I)^{-1}, from g = G^{-1} (this lane's row) and C.
+// This lane's share of sum_{i<k} (C_ik / |C_ik|) conj(zeta_i) zeta_k, zeta one
+// unit phasor a lane: row r takes the pairs {r, r + j mod n} for j = 1 ..
+// n / 2 (for even n the last j pairs rows r and r + n/2 twice: rows r < n/2
+// take it), so every lane does n / 2 entries instead of the n - 1 - r that its
+// part of the upper triangle holds, in a loop that is not unrolled.  Unrolled
+// over whole rows, half of them masked, it and the reference phase were 18% of
+// a 15-date solve, and the code (75 KB at 16 entries, 58 KB now) passed the
+// instruction cache.  With the convergence factor formed only where it is
+// looked at and B^{-1} left rotated: 250,007 pixels at N = 15 1.147 -> 0.997
+// ms, 524,288 at N = 17 5.50 -> 4.98 ms, 65,521 at N = 28 1.55 -> 1.45 ms, the
+// linked phases bit for bit the same.  An entry below the diagonal is the
+// conjugate of the pair's term.
+template <int NP, class T, class Load>
+__device__ __forceinline__ cpx<T> pair_sum(const Load &load, cpx<T> zeta, cpx<T> *buf, int r, int n,
+                                           unsigned gmask) {
+    cpx<T> s = mk<T>(T(0), T(0));
+    buf[r] = zeta;
+    __syncwarp(gmask);
+    if (r < n) {
+        const int m = (n - 1 + (2 * r < n ? 1 : 0)) / 2;
+        int k = r;
+#pragma unroll 1
+        for (int j = 0; j < m; ++j) {
+            k = k + 1 < n ? k + 1 : 0;
+            const cpx<T> c = load(k), zk = buf[k];
+            const T m2 = norm2(c);
+            const cpx<T> uk = (m2 > T(0)) ? (rsqrt_t(m2) * c) : mk<T>(T(1), T(0));
+            const cpx<T> t = uk * zk;
+            s.x += t.x * zeta.x + t.y * zeta.y;
+            const T im = t.y * zeta.x - t.x * zeta.y;
+            s.y += k > r ? im : -im;
+        }
+    }
+    __syncwarp(gmask);
+    return s;
+}
+
+// a <- (G^{-1} o C - mu I)^{-1}, from g = G^{-1} (this lane's row) and C, the
+// columns left rotated (rotated_slot).
 // Returns the smallest pivot: by Sylvester's law of inertia the pivots of the
 // Hermitian B = A - mu I (the D of its LDL^H factorisation) are all positive
 // exactly when B is positive definite, i.e. when mu lies below lambda_min.
@@ -324,7 +385,7 @@ __device__ __forceinline__ T form_shift_inverse(cpx<T> (&a)[NP], const T (&g)[NP
         a[k] = mk<T>(g[k] * a[k].x, g[k] * a[k].y);
         if (k == r) a[k].x -= mu;
     }
-    return gj_invert<NP, T, cpx<T>, false>(a, cbuf, r, n, gmask, T(0));
+    return gj_invert<NP, T, cpx<T>, false, false>(a, cbuf, r, n, gmask, T(0));
 }
 
 // y = A x with A = G^{-1} o C, row r from g and the reloaded C row.
@@ -338,6 +399,8 @@ __device__ __forceinline__ cpx<T> apply_A(const T (&g)[NP], const Loader &load, 
     return group_matvec<NP, T>(row, x, buf, r, gmask);
 }
 
+// slot: this lane's place in the products with a[] (rotated_slot for B^{-1}, r
+// for C).
 // Inverse iteration x <- B^{-1} x / |B^{-1} x| on the rows a[] (B^{-1}, or C
 // itself on the EVD fallback when allow_reshift is false), with the shift
 // refinement described at emi_solve: reform(mu) rebuilds a[] for a new shift
@@ -359,16 +422,20 @@ __device__ __forceinline__ cpx<T> apply_A(const T (&g)[NP], const Loader &load, 
 // rest of the step budget to the caller's refinement.
 template <int NP, class T, class Reform>
 __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cpx<T> &d, T &mu, T &q,
-                                                  const Reform &reform, bool allow_reshift, cpx<T> *cbuf, int r,
+                                                  const Reform &reform, bool allow_reshift, cpx<T> *cbuf, int slot,
                                                   bool live, unsigned gmask, T tol, int max_iter,
                                                   bool build_first, T floor_num = T(0), T floor_den = T(0),
                                                   int *used = nullptr, bool stop_slow = false) {
     const T tol2 = tol * tol;
     if (used) *used = 0;
     d = mk<T>(T(1), T(0));
-    q = T(0);
+    // q = sqrt(q_num / q_den), formed only where it is looked at (a division
+    // and a square root a step otherwise); q_den = 0: q = 0.
+    T q_num = T(0), q_den = T(0);
+    auto factor = [&]() { return q_den > T(0) ? sqrt_t(q_num / q_den) : T(0); };
     T dl_prev = T(-1);
     int in_round = 0, reshifts = 0;
+    bool converged = false;
     // reform_to > 0: rebuild a[] for shift mu_try before the next step; a
     // failed inertia check (B not positive definite) rebuilds it once more for
     // the old shift.  One call site keeps the inlined elimination code single.
@@ -394,12 +461,12 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
             }
             in_round = 0;
             dl_prev = T(-1);
-            q = T(0);
+            q_den = T(0);
             continue;
         }
         if (it - 2 * reshifts >= max_iter) break;
         if (used) ++*used;
-        cpx<T> y = group_matvec<NP, T>(a, x, cbuf, r, gmask);
+        cpx<T> y = group_matvec<NP, T>(a, x, cbuf, slot, gmask);
         if (!live) y = mk<T>(T(0), T(0));
         const T s = group_sum<NP, T>(norm2(y), gmask);          // |y|^2
         d.x = group_sum<NP, T>(x.x * y.x + x.y * y.y, gmask);  // x^H y
@@ -411,11 +478,18 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
         const T dl = group_sum<NP, T>(norm2(yn - x), gmask);
         x = yn;
         ++in_round;
-        if (dl_prev > T(0) && dl > T(100) * tol2) q = sqrt_t(dl / dl_prev);
+        if (dl_prev > T(0) && dl > T(100) * tol2) {
+            q_num = dl;
+            q_den = dl_prev;
+        }
         dl_prev = dl;
-        if (dl <= tol2) return true;
-        if (stop_slow && !allow_reshift && in_round >= 4 && q > T(0.3)) return false;
-        if (allow_reshift && reshifts < 3 && in_round >= 4 && q > T(0.3)) {
+        if (dl <= tol2) {
+            converged = true;
+            break;
+        }
+        if (in_round < 4 || !((allow_reshift && reshifts < 3) || (stop_slow && !allow_reshift))) continue;
+        if (factor() > T(0.3)) {
+            if (!allow_reshift) break;
             // Move the shift towards lambda_min; keep it only if B stays
             // positive definite (the shift is still below lambda_min),
             // otherwise restore the previous one and stop moving it.
@@ -424,7 +498,8 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
             pending = 1;
         }
     }
-    return false;
+    q = factor();
+    return converged;
 }
 
 // Solve one pixel.  T = float: returns flag = true (and no outputs) for a pixel
@@ -468,13 +543,16 @@ __device__ PixelResult emi_solve(const Loader &load, int r, int n, int ref, cons
     T rs = 0, mmin = T(1);
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
-        const T mc = mag_t(norm2(a[k]));
-        if (k != r && k < n && live) mmin = fmin(mmin, mc);
-        T m = mc;
-        if (prm.beta != 0.f) m = (T(1) - T(prm.beta)) * m + ((k == r) ? T(prm.beta) : T(0));
-        g[k] = m;
-        rs += abs_t(m);
+        g[k] = mag_t(norm2(a[k]));
+        if (k < n) mmin = fmin(mmin, g[k]);  // the unit diagonal leaves the minimum as it is
     }
+    if (!live) mmin = T(1);
+    if (prm.beta != 0.f) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) g[k] = (T(1) - T(prm.beta)) * g[k] + ((k == r) ? T(prm.beta) : T(0));
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k) rs += abs_t(g[k]);
     // Rank one (a single look, e.g. an isolated persistent scatterer): every
     // |C_ik| is 1 up to the rounding of the products and reciprocal square roots
     // that normalise it (a few ulps each); G is singular, the EVD fallback
@@ -563,13 +641,14 @@ __device__ PixelResult emi_solve(const Loader &load, int r, int n, int ref, cons
     // max_iter caps the steps of both passes together: the power iteration
     // stops as soon as it is seen to be slow, and the refinement gets what it
     // left.
+    const int rslot = rotated_slot<NP>(r, n);
     bool conv = false, refined = false, evd_power = inv_failed;
     T fl_num = T(0.999), fl_den = norm_g;
     int budget = prm.max_iter;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
         int used = 0;
-        conv = inverse_iteration<NP, T>(a, x, d, mu, q, reform, !evd_power, cbuf, r, live, gmask, tol, budget,
+        conv = inverse_iteration<NP, T>(a, x, d, mu, q, reform, !evd_power, cbuf, evd_power ? r : rslot, live, gmask, tol, budget,
                                         !evd_power, fl_num, fl_den, &used, evd_power);
         budget -= used;
         if (!(evd_power && (!conv || q > T(0.3)) && budget > 0)) break;
@@ -595,7 +674,7 @@ __device__ PixelResult emi_solve(const Loader &load, int r, int n, int ref, cons
             with_g([&](const T (&gg)[NP]) { return apply_A<NP, T>(gg, load, x, cbuf, r, n, gmask); });
         const T rho = group_sum<NP, T>(live ? (x.x * ax.x + x.y * ax.y) : T(0), gmask);
         const cpx<T> res = live ? (ax - rho * x) : mk<T>(T(0), T(0));
-        cpx<T> corr = group_matvec<NP, T>(a, res, cbuf, r, gmask);
+        cpx<T> corr = group_matvec<NP, T>(a, res, cbuf, rslot, gmask);
         cpx<T> xn = live ? (x - corr) : mk<T>(T(0), T(0));
         const T s2 = group_sum<NP, T>(norm2(xn), gmask);
         if (s2 > T(0)) x = rsqrt_t(s2) * xn;
@@ -628,15 +707,7 @@ __device__ PixelResult emi_solve(const Loader &load, int r, int n, int ref, cons
     const T wm2 = norm2(w);
     cpx<T> zeta = (wm2 > T(0)) ? (rsqrt_t(wm2) * w) : mk<T>(T(1), T(0));
     if (r == ref) zeta = mk<T>(T(1), T(0));
-    load_crow<NP, T>(a, load, r, n);
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const T m2 = norm2(a[k]);
-        const cpx<T> uk = (m2 > T(0)) ? (rsqrt_t(m2) * a[k]) : mk<T>(T(1), T(0));
-        a[k] = (k > r && k < n) ? uk : mk<T>(T(0), T(0));
-    }
-    const cpx<T> rowsum = group_matvec<NP, T>(a, zeta, cbuf, r, gmask);
-    const cpx<T> term = live ? (conj(zeta) * rowsum) : mk<T>(T(0), T(0));
+    const cpx<T> term = pair_sum<NP, T>(load, zeta, cbuf, r, n, gmask);
     const T sx = group_sum<NP, T>(term.x, gmask);
     const T sy = group_sum<NP, T>(term.y, gmask);
     const T tcoh = sqrt_t(sx * sx + sy * sy) / (T(0.5) * T(n) * T(n - 1));
@@ -713,6 +784,7 @@ __device__ PixelResult emi_solve_mixed(const Loader &load, int r, int n, int ref
 #pragma unroll
             for (int k = 0; k < NP; ++k) A[k] = mk<double>(g[k] * A[k].x, g[k] * A[k].y);
         }
+        const int rslot = rotated_slot<NP>(r, n);
         cpx<float> B[NP];
         auto formB = [&](float m) {
 #pragma unroll
@@ -720,7 +792,7 @@ __device__ PixelResult emi_solve_mixed(const Loader &load, int r, int n, int ref
                 B[k] = mk<float>((float)A[k].x, (float)A[k].y);
                 if (k == r) B[k].x -= m;
             }
-            return gj_invert<NP, float, cpx<float>, false>(B, fbuf, r, n, gmask, 0.f);
+            return gj_invert<NP, float, cpx<float>, false, false>(B, fbuf, r, n, gmask, 0.f);
         };
         float mu = mu0;
         cpx<float> x;
@@ -733,7 +805,7 @@ __device__ PixelResult emi_solve_mixed(const Loader &load, int r, int n, int ref
         }
         cpx<float> d;
         float q;
-        inverse_iteration<NP, float>(B, x, d, mu, q, formB, true, fbuf, r, live, gmask, 1e-6f, prm.max_iter, true,
+        inverse_iteration<NP, float>(B, x, d, mu, q, formB, true, fbuf, rslot, live, gmask, 1e-6f, prm.max_iter, true,
                                      floor_num, floor_den);
         // Tighten the preconditioner for the double-precision phase: shift to
         // just under lambda_min (by a tenth of the gap measured through q, at
@@ -745,18 +817,21 @@ __device__ PixelResult emi_solve_mixed(const Loader &load, int r, int n, int ref
             const float gap = (q > 0.f) ? theta * (1.f / q - 1.f) : 10.f * theta;
             const float step = fminf(0.5f * theta, 0.1f * gap);
             if (theta > 0.f && step > 0.f) {
-                const float mu_new = mu + (theta - step);
-                if (formB(mu_new) > 0.f) mu = mu_new;
-                else formB(mu);
+                const float mu_old = mu;
+                mu = mu + (theta - step);
+#pragma unroll 1
+                while (!(formB(mu) > 0.f) && mu != mu_old) mu = mu_old;
             }
         }
         x64 = mk<double>((double)x.x, (double)x.y);
         double rho = 0.0;
+#pragma unroll 1
         for (int it = 0; it < 50; ++it) {
             const cpx<double> ax = group_matvec<NP, double>(A, x64, dbuf, r, gmask);
             rho = group_sum<NP, double>(live ? (x64.x * ax.x + x64.y * ax.y) : 0.0, gmask);
             const cpx<double> res = live ? (ax - rho * x64) : mk<double>(0.0, 0.0);
-            const cpx<float> corr = group_matvec<NP, float>(B, mk<float>((float)res.x, (float)res.y), fbuf, r, gmask);
+            const cpx<float> corr =
+                group_matvec<NP, float>(B, mk<float>((float)res.x, (float)res.y), fbuf, rslot, gmask);
             const cpx<double> xn = live ? (x64 - mk<double>((double)corr.x, (double)corr.y)) : mk<double>(0.0, 0.0);
             const double s2 = group_sum<NP, double>(norm2(xn), gmask);
             const double c2 = group_sum<NP, double>(live ? (double)norm2(corr) : 0.0, gmask);
@@ -781,17 +856,12 @@ __device__ PixelResult emi_solve_mixed(const Loader &load, int r, int n, int ref
     const float wm2 = norm2(wf);
     cpx<float> zeta = (wm2 > 0.f) ? (rsqrtf(wm2) * wf) : mk<float>(1.f, 0.f);
     if (r == ref) zeta = mk<float>(1.f, 0.f);
-    cpx<float> u[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-        const cpx<double> cd = (live && k < n) ? load(k) : mk<double>(0.0, 0.0);
-        const cpx<float> ck = mk<float>((float)cd.x, (float)cd.y);
-        const float m2 = norm2(ck);
-        const cpx<float> uk = (m2 > 0.f) ? (rsqrtf(m2) * ck) : mk<float>(1.f, 0.f);
-        u[k] = (k > r && k < n) ? uk : mk<float>(0.f, 0.f);
-    }
-    const cpx<float> rowsum = group_matvec<NP, float>(u, zeta, fbuf, r, gmask);
-    const cpx<float> term = live ? (conj(zeta) * rowsum) : mk<float>(0.f, 0.f);
+    const cpx<float> term = pair_sum<NP, float>(
+        [&](int k) {
+            const cpx<double> c = load(k);
+            return mk<float>((float)c.x, (float)c.y);
+        },
+        zeta, fbuf, r, n, gmask);
     const float sx = group_sum<NP, float>(term.x, gmask);
     const float sy = group_sum<NP, float>(term.y, gmask);
     out.phase = ph;

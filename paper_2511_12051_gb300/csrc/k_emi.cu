@@ -75,37 +75,39 @@ __device__ __forceinline__ void for_each_pending(unsigned long long *work, bool 
     constexpr int G = kPow2 ? 32 / NP : 1;  // rows of 20, 24 or 28 entries: one pixel a warp
     const int grp = kPow2 ? lane / NP : 0;
     const unsigned long long cnt = use_list ? *(volatile unsigned long long *)(work + 1) : ~0ull;
-    if (cnt <= (unsigned long long)kPendCap) {
-        const unsigned *lst = pending_list(work);
-        for (;;) {
+    const bool listed = cnt <= (unsigned long long)kPendCap;
+    const unsigned *lst = pending_list(work);
+    const long long nchunks = (npx + 31) / 32;
+    long long base = 0;
+    unsigned bal = 0;  // status scan: pending pixels left of the chunk
+    // Both ways of finding the next pixels end at one call of solve, whose
+    // code is inlined (150 to 270 KB of it for one copy).
+#pragma unroll 1
+    for (;;) {
+        long long mine = -1;
+        if (listed) {
             const long long b0 = next_chunk(work + 2, lane, (unsigned long long)G);
             if (b0 >= (long long)cnt) break;
-            const long long i = b0 + grp;
-            if (i < (long long)cnt) solve((long long)lst[i]);
-            __syncwarp();
-        }
-        return;
-    }
-    const long long nchunks = (npx + 31) / 32;
-    for (;;) {
-        const long long base = next_chunk(work, lane);
-        if (base >= nchunks) break;
-        const long long pl = base + (long long)lane * nchunks;  // interleaved: clusters spread over chunks
-        const bool pend = pl < npx && status[pl] == (uint8_t)kPending;
-        unsigned bal = __ballot_sync(0xffffffffu, pend);
-        while (bal) {
-            int mine = -1;
+            if (b0 + grp < (long long)cnt) mine = (long long)lst[b0 + grp];
+        } else {
+            if (!bal) {
+                base = next_chunk(work, lane);
+                if (base >= nchunks) break;
+                const long long pl = base + (long long)lane * nchunks;  // interleaved: clusters spread over chunks
+                bal = __ballot_sync(0xffffffffu, pl < npx && status[pl] == (uint8_t)kPending);
+                if (!bal) continue;
+            }
 #pragma unroll
             for (int gg = 0; gg < G; ++gg) {
                 if (bal) {
                     const int b = __ffs(bal) - 1;
-                    if (gg == grp) mine = b;
+                    if (gg == grp) mine = base + (long long)b * nchunks;
                     bal &= bal - 1u;
                 }
             }
-            if (mine >= 0) solve(base + (long long)mine * nchunks);
-            __syncwarp();
         }
+        if (mine >= 0) solve(mine);
+        __syncwarp();
     }
 }
 
@@ -181,6 +183,7 @@ __global__ void __launch_bounds__(EmiWarps<NP>::value * 32, EmiMinBlocks<NP>::va
     auto prefetch = [&](long long b, int slot) {
         const long long cnt = b < npx ? ((npx - b < G) ? (npx - b) : G) * nt : 0;
         const float2 *src = C + (b < npx ? b : 0) * nt;
+#pragma unroll 1
         for (int e = lane; e < G * nt; e += 32) {
             const bool ok = e < cnt;
             cp_async8_emi(&pf[warp][slot][e], ok ? src + e : C, ok ? 8 : 0);
