@@ -76,10 +76,10 @@ struct AdjShared {
     static constexpr int oBuf = oC + (NP + 1) * kPitch * 8;
     static constexpr int oV = oBuf + kBuf;
     static constexpr int oRs = oV + kLanes * 8;
-    static constexpr int oM = oRs + kLanes * 4;  // two float matrices: the G^-1 row slots, then products
-    static constexpr int oG = oM + 2 * kMat;     // G^-1 [k][r]
-    static_assert(2 * kMat >= kLanes * (NP + 4) * 4, "the G^-1 row slots fit the product matrices");
-    static_assert(oM % 16 == 0 && kMat % 16 == 0, "16-byte loads");
+    static constexpr int oG = oRs + kLanes * 4;  // G^-1 [k][r], then [r][k]; k_adj_prep: the solve's G^-1 row slots
+    static constexpr int oM = oG + 2 * kMat;     // k_adj_pixel: R [r][k], then T [k][r], then GG [r][k]
+    static_assert(2 * kMat >= kLanes * (NP + 4) * 4, "the G^-1 row slots fit");
+    static_assert(oG % 16 == 0 && kMat % 16 == 0, "16-byte loads");
     char *base;
     __device__ __forceinline__ cpx<float> *C() const { return reinterpret_cast<cpx<float> *>(base + oC); }
     __device__ __forceinline__ cpx<float> *buf() const { return reinterpret_cast<cpx<float> *>(base + oBuf); }
@@ -87,6 +87,7 @@ struct AdjShared {
     __device__ __forceinline__ float *rs() const { return reinterpret_cast<float *>(base + oRs); }
     __device__ __forceinline__ float *M() const { return reinterpret_cast<float *>(base + oM); }
     __device__ __forceinline__ float *g() const { return reinterpret_cast<float *>(base + oG); }
+    __device__ __forceinline__ float *grow() const { return reinterpret_cast<float *>(base + oG + kMat); }
 };
 
 // Lane numbering of a group.
@@ -104,84 +105,78 @@ struct AdjLane {
     }
 };
 
-// C <- the padded Hermitian matrix of the packed triangle: row i of the
-// triangle is read by consecutive lanes and written as row and column i.
+// C <- the padded Hermitian matrix of the packed triangle, unit diagonal: row i
+// of the triangle is read by consecutive lanes and written as row and column i.
 template <int NP>
-__device__ __forceinline__ void adj_load(const AdjShared<NP> &sh, const float2 *__restrict__ Cpix, int r, int n) {
+__device__ __forceinline__ void adj_load(const AdjShared<NP> &sh, const float2 *Cpix, int r, int n) {
     constexpr int P = AdjShared<NP>::kPitch;
     cpx<float> *C = sh.C();
 #pragma unroll 4
     for (int i = 0; i < NP; ++i) {
         if (r < i || r >= NP) continue;
-        float2 c = make_float2(i == r && i >= n ? 1.f : 0.f, 0.f);
-        if (r < n) c = __ldg(Cpix + packed_index(n, i, r));
+        float2 c = make_float2(i == r ? 1.f : 0.f, 0.f);
+        if (r < n && r > i) c = Cpix[packed_index(n, i, r)];
         C[i * P + r] = mk<float>(c.x, c.y);
         if (r > i) C[r * P + i] = mk<float>(c.x, -c.y);
     }
     if (r < NP) C[NP * P + r] = mk<float>(0.f, 0.f);
 }
 
-// Per-pixel part of the adjoint: solves the pixel (v into shared memory), puts
-// G^-1 into shared memory (1 between live dates on the EVD fallback) and
-// leaves this lane's row of M = (A - lambda I + c v v^H)^-1 in mrow.  G^-1 is
-// the one that the solve leaves in its row slots.  Dates without power
-// (S_kk = 0) carry no gradient: their rows and columns of g are 0.
-template <int NP>
+// A prepared pixel (k_adj_prep): this lane's entry of the eigenvector and
+// 1 / sqrt(S_rr) (0 where S_rr = 0), the eigenvalue, and max(1, |lambda|).
 struct AdjPixel {
     cpx<float> v;
-    float rsr, cdef;
+    float rsr, lam, cdef;
     bool evd, live;
 };
-
 template <int NP>
-__device__ __forceinline__ void adj_prepare(AdjPixel<NP> &S, cpx<float> (&mrow)[NP], const AdjShared<NP> &sh,
-                                            const AdjLane<NP> &L, const float *__restrict__ Sd, long long p, int n,
-                                            int ref, const EmiParams &q) {
-    constexpr int P = AdjShared<NP>::kPitch;
-    const int r = L.r;
-    const unsigned gmask = L.gmask;
-    cpx<float> *cbuf = sh.buf();
-    const AdjRow<NP> ld{sh.C() + (r < NP ? r : NP) * P};
-    float *gslot = sh.M() + r * (NP + 4);
+__device__ __forceinline__ AdjPixel adj_read(const AdjShared<NP> &sh, int r, int n, const float2 *Cpix,
+                                             const float *Sdp, const float2 *Hp) {
+    AdjPixel S;
     S.live = r < n;
-    const PixelResult res =
-        emi_solve<NP, float, AdjRow<NP>, true>(ld, r, n, ref, q, cbuf, gmask, L.glane0, false, gslot);
-    S.evd = res.evd;
-    S.v = S.live ? res.v : mk<float>(0.f, 0.f);
-    const float sr = S.live ? __ldg(Sd + p * n + r) : 0.f;
-    S.rsr = sr > 0.f ? rsqrtf(sr) : 0.f;
+    S.v = S.live ? mk<float>(Sdp[r], Cpix[packed_index(n, r, r)].y) : mk<float>(0.f, 0.f);
+    S.rsr = S.live ? Hp[r].x : 0.f;
+    S.lam = Cpix[0].x;
+    S.evd = Hp[0].y != 0.f;
+    S.cdef = fmaxf(1.f, fabsf(S.lam));
     sh.v()[r] = S.v;
     sh.rs()[r] = S.rsr;
-    __syncwarp(gmask);
-    // A row (C, or G^-1 o C) into mrow, the masked G^-1 row into [k][r].
+    return S;
+}
+
+// mrow: this lane's row of (A - lambda I + c v v^H)^-1 (c keeps the deflated
+// matrix well scaled); G^-1 (1 on the EVD fallback) into sh.g(), where a lane
+// reads its own row, and sh.grow(), where all lanes read one row.  G can be
+// conditioned up to 1e6, and its computed inverse is then symmetric to 0.1 only,
+// so the two are not interchangeable: the products keep the order G^-1 R, then
+// (G^-1 R) G^-1, each over rows.
+template <int NP>
+__device__ __forceinline__ void adj_invert(const AdjPixel &S, cpx<float> (&mrow)[NP], const AdjShared<NP> &sh,
+                                           const AdjLane<NP> &L, int n, float beta) {
+    const int r = L.r;
+    const AdjRow<NP> ld{sh.C() + (r < NP ? r : NP) * AdjShared<NP>::kPitch};
+    ld.all(mrow);
+    float gi[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) gi[k] = mag_t(norm2(mrow[k]));
+    if (beta != 0.f) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) gi[k] = (1.f - beta) * gi[k] + ((k == r) ? beta : 0.f);
+    }
+    if (!S.evd) gj_invert<NP, float, float, true>(gi, reinterpret_cast<float *>(sh.buf()), r, n, L.gmask, 0.f);
     ld.all(mrow);
 #pragma unroll
-    for (int q4 = 0; q4 < NP / 4; ++q4) {
-        const float4 g4 = reinterpret_cast<const float4 *>(gslot)[q4];
-        const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int k = q4 * 4 + e;
-            const float gk = S.evd ? 1.f : gg[e];
-            mrow[k] = mk<float>(gk * mrow[k].x, gk * mrow[k].y);
-            if (r < NP) sh.g()[k * NP + r] = S.rsr > 0.f && sh.rs()[k] > 0.f ? gk : 0.f;
-        }
-    }
-    // lambda = v^H A v (the eigenvalue the perturbation is about)
-    const cpx<float> av = group_matvec<NP, float>(mrow, S.v, cbuf, r, gmask);
-    const float lam = group_sum<NP, float>(S.live ? (S.v.x * av.x + S.v.y * av.y) : 0.f, gmask);
-    // c keeps the deflated matrix well scaled, with the sign that leaves it
-    // definite (A - lambda I is positive semidefinite, on the EVD fallback
-    // negative: lambda is the largest eigenvalue of C), so that the inversion
-    // without pivoting meets no zero pivot (a single look and four dates did)
-    S.cdef = S.evd ? -fmaxf(1.f, fabsf(lam)) : fmaxf(1.f, fabsf(lam));
-    const cpx<float> cv = S.cdef * S.v;
-#pragma unroll
     for (int k = 0; k < NP; ++k) {
-        mrow[k] = mrow[k] + cv * conj(sh.v()[k]);
-        if (k == r && S.live) mrow[k].x -= lam;
+        if (S.evd) gi[k] = 1.f;
+        if (r < NP) sh.g()[k * NP + r] = gi[k];
+        // A's entry is rounded before the deflation is added (not contracted
+        // with it): its gap can be small, and A is what lambda was formed with.
+        mrow[k] = mk<float>(__fmul_rn(gi[k], mrow[k].x), __fmul_rn(gi[k], mrow[k].y));
+        mrow[k] = mrow[k] + S.cdef * (S.v * conj(sh.v()[k]));
+        if (k == r && S.live) mrow[k].x -= S.lam;
     }
-    gj_invert<NP, float, cpx<float>, false>(mrow, cbuf, r, n, gmask, 0.f);
+    if (r < NP) store_row<NP>(sh.grow() + r * NP, gi);
+    gj_invert<NP, float, cpx<float>, false>(mrow, sh.buf(), r, n, L.gmask, 0.f);
 }
 
 }  // namespace
@@ -211,19 +206,16 @@ __global__ void __launch_bounds__(256) k_adj_sdiag(const __grid_constant__ Plane
     }
 }
 
-// Per output pixel: H_p from the coherence C (packed), the diagonal sums and
-// the phase weights w [n][npx].  Pixels without data get H_p = 0.  With
-// K = GC + GC^H off the diagonal, H_rk = K_rk / sqrt(S_rr S_kk) and H_rr =
-// -sum_k Re(conj(K_rk) C_rk) / S_rr; K_rk = -g_rk (u_r conj(v_k) + v_r conj(u_k))
-// + (1 - beta) (GG_rk + GG_kr) C_rk / |C_rk|.
-// What bounds it is instruction issue and fetch: a pixel is two eliminations
-// and two products of N x N matrices by one warp.  The products used to be
-// unrolled over both indices, 576 to 1024 multiply-adds of straight-line code
-// each that every warp fetched for itself, in rows of 24 or 32 entries; as
-// loops over the rows, in rows of 20 to 32 entries in steps of 4, with G^-1
-// taken from the solve instead of inverted again, 301 x 403 pixels at stride 1
-// take 2.88 instead of 5.36 ms at N = 20, 7.6 instead of 12.4 ms at N = 28 and
-// 0.99 instead of 1.38 ms at N = 14.
+// The adjoint runs in two kernels: this one solves the pixel (the single-
+// precision solve is what the adjoint differentiates), a second one forms what
+// depends on the weights.  One kernel of both (110 to 190 KB of code, most of it
+// the solve's) lost a third of its issue slots to instruction fetch.  Per output
+// pixel, in place of what it has read: Sd: Re v;  C: Im v in the imaginary part
+// of the diagonal, lambda = v^H A v (the eigenvalue that the perturbation is
+// about) in the real part of its first entry;  H area: 1 / sqrt(S_kk) (0 where
+// S_kk = 0) in its first n entries, whether the EVD fallback solved the pixel in
+// the first imaginary part.  Pixels without data stay as they are (NaN on C's
+// diagonal).
 constexpr int kAdjWarps = 2;
 
 template <int NP>
@@ -233,11 +225,84 @@ struct AdjMinBlocks {
 
 template <int NP>
 __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
-    k_adj_pixel(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref,
-                const EmiParams prm, const float *__restrict__ w, float2 *__restrict__ Hout) {
+    k_adj_prep(float2 *C, float *Sd, int n, long long npx, int ref, const EmiParams prm, float2 *__restrict__ Hout) {
     using Sh = AdjShared<NP>;
     constexpr int G = Sh::G, P = Sh::kPitch;
-    constexpr int kBytes = Sh::oG + Sh::kMat;
+    __shared__ __align__(16) char smem[kAdjWarps * G * Sh::oM];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const AdjLane<NP> L(lane);
+    const int r = L.r, grp = L.glane0 / NP;
+    const unsigned gmask = L.gmask;
+    const Sh sh{smem + (warp * G + grp) * Sh::oM};
+    cpx<float> *cbuf = sh.buf();
+    const AdjRow<NP> ld{sh.C() + (r < NP ? r : NP) * P};
+    float *gslot = sh.g() + r * (NP + 4);
+    const bool live = r < n;
+    const long long nt = ntri(n);
+    const long long step = (long long)gridDim.x * kAdjWarps * G;
+    EmiParams q = prm;
+    q.fp64_resolve = 0;
+
+    for (long long base = ((long long)blockIdx.x * kAdjWarps + warp) * G; base < npx; base += step) {
+        const long long p = base + grp;
+        const bool valid = p < npx;
+        float2 *Cpix = C + (valid ? p : 0) * nt;
+        bool nan = false;
+        if (valid && live) nan = isnan(Cpix[packed_index(n, r, r)].x);
+        nan = __any_sync(gmask, nan);
+        if (!valid || nan) continue;
+        adj_load<NP>(sh, Cpix, r, n);
+        __syncwarp(gmask);
+        const PixelResult res =
+            emi_solve<NP, float, AdjRow<NP>, true>(ld, r, n, ref, q, cbuf, gmask, L.glane0, false, gslot);
+        const cpx<float> v = live ? res.v : mk<float>(0.f, 0.f);
+        // A row: C, or G^-1 o C with the G^-1 row that the solve left in its slot
+        cpx<float> m[NP];
+        ld.all(m);
+        if (!res.evd) {
+#pragma unroll
+            for (int q4 = 0; q4 < NP / 4; ++q4) {
+                const float4 g4 = reinterpret_cast<const float4 *>(gslot)[q4];
+                const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int k = q4 * 4 + e;
+                    m[k] = mk<float>(gg[e] * m[k].x, gg[e] * m[k].y);
+                }
+            }
+        }
+        const cpx<float> av = group_matvec<NP, float>(m, v, cbuf, r, gmask);
+        const float lam = group_sum<NP, float>(live ? (v.x * av.x + v.y * av.y) : 0.f, gmask);
+        if (live) {
+            const float sr = Sd[p * n + r];
+            Sd[p * n + r] = v.x;
+            Hout[p * nt + r] = make_float2(sr > 0.f ? rsqrtf(sr) : 0.f, res.evd ? 1.f : 0.f);
+            Cpix[packed_index(n, r, r)] = make_float2(r == 0 ? lam : 1.f, v.y);
+        }
+        __syncwarp(gmask);
+    }
+}
+
+// Per output pixel: H_p from the coherence C (packed), the diagonal sums and
+// the phase weights w [n][npx].  Pixels without data get H_p = 0.  With
+// K = GC + GC^H off the diagonal, H_rk = K_rk / sqrt(S_rr S_kk) and H_rr =
+// -sum_k Re(conj(K_rk) C_rk) / S_rr; K_rk = -g_rk u_r conj(v_k) - g_kr v_r conj(u_k)
+// + (1 - beta) (GG_rk + GG_kr) C_rk / |C_rk|.
+// What bounds it is instruction issue and fetch: a pixel is two eliminations
+// and two products of N x N matrices by one warp.  The products used to be
+// unrolled over both indices, 576 to 1024 multiply-adds of straight-line code
+// each that every warp fetched for itself, in rows of 24 or 32 entries.  As
+// loops over the rows, in rows of 20 to 32 entries in steps of 4, apart from
+// the solve (k_adj_prep), 301 x 403 pixels at stride 1 take 2.55 ms in both
+// kernels instead of 5.36 at N = 20, 5.9 instead of 12.4 at N = 28 and 0.95
+// instead of 1.38 at N = 14.
+template <int NP>
+__global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
+    k_adj_pixel(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref,
+                float beta, const float *__restrict__ w, float2 *Hout) {
+    using Sh = AdjShared<NP>;
+    constexpr int G = Sh::G, P = Sh::kPitch;
+    constexpr int kBytes = Sh::oM + Sh::kMat;
     __shared__ __align__(16) char smem[kAdjWarps * G * kBytes];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const AdjLane<NP> L(lane);
@@ -246,8 +311,6 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
     const Sh sh{smem + (warp * G + grp) * kBytes};
     const long long nt = ntri(n);
     const long long step = (long long)gridDim.x * kAdjWarps * G;
-    EmiParams q = prm;
-    q.fp64_resolve = 0;  // the adjoint differentiates the single-precision solve
 
     for (long long base = ((long long)blockIdx.x * kAdjWarps + warp) * G; base < npx; base += step) {
         const long long p = base + grp;
@@ -265,26 +328,28 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
         }
         adj_load<NP>(sh, Cpix, r, n);
         __syncwarp(gmask);
-        AdjPixel<NP> S;
+        float2 *Hp = Hout + p * nt;  // what k_adj_prep left; H at the end
+        const AdjPixel S = adj_read<NP>(sh, r, n, Cpix, Sd + p * n, Hp);
+        __syncwarp(gmask);
         cpx<float> u;
         {
             cpx<float> mrow[NP];
-            adj_prepare<NP>(S, mrow, sh, L, Sd, p, n, ref, q);
+            adj_invert<NP>(S, mrow, sh, L, n, beta);
             // Gradient on v (gauge-free), projected orthogonal to v.
             const float wr = live ? __ldg(w + (long long)r * npx + p) : 0.f;
             const float wsum = group_sum<NP, float>(live && r != ref ? wr : 0.f, gmask);
-            const float m2 = norm2(S.v);
+            const float m2 = __fmaf_rn(S.v.x, S.v.x, __fmul_rn(S.v.y, S.v.y));
             const float coef = (r == ref) ? -wsum : wr;
             cpx<float> gv = (live && m2 > 0.f) ? (coef / m2) * mk<float>(-S.v.y, S.v.x) : mk<float>(0.f, 0.f);
             const cpx<float> t = conj(S.v) * gv;
             const float sx = group_sum<NP, float>(t.x, gmask), sy = group_sum<NP, float>(t.y, gmask);
             gv = gv - S.v * mk<float>(sx, sy);
-            // u = M g_v  (orthogonal to v)
+            // u = (A - lambda I + c v v^H)^-1 g_v  (orthogonal to v)
             u = group_matvec<NP, float>(mrow, gv, sh.buf(), r, gmask);
         }
         cpx<float> *uall = sh.buf();
         const cpx<float> *Crow = sh.C() + rr * P, *vg = sh.v();
-        const float *gcol = sh.g() + rr;
+        const float *gcol = sh.g() + rr, *gtr = sh.grow() + rr;
         uall[r] = u;
         float GG[NP];
 #pragma unroll
@@ -295,9 +360,9 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
             // unrolled over the row index (short code), the left factor's
             // entry read from shared memory and the right factor's row as
             // broadcast 16-byte loads.
-            float *R = sh.M(), *T = sh.M() + NP * NP;
+            float *R = sh.M(), *T = R;
             if (r < NP) {
-                float rrow[NP];  // -R
+                float rrow[NP];
 #pragma unroll
                 for (int k = 0; k < NP; k += 2) {
                     cpx<float> c[2], v[2];
@@ -305,8 +370,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
                     load_pair(vg + k, v);
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const cpx<float> t = c[e] * v[e];
-                        rrow[k + e] = u.x * t.x + u.y * t.y;
+                        const cpx<float> ga = mk<float>(0.f, 0.f) - u * conj(v[e]);
+                        rrow[k + e] = ga.x * c[e].x + ga.y * c[e].y;
                     }
                 }
                 store_row<NP>(R + rr * NP, rrow);
@@ -325,6 +390,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
                     GG[q4 * 4 + 3] += gj * x.w;
                 }
             }
+            __syncwarp(gmask);
             if (r < NP) {
 #pragma unroll
                 for (int k = 0; k < NP; ++k) T[k * NP + rr] = GG[k];
@@ -334,22 +400,22 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
 #pragma unroll 2
             for (int j = 0; j < n; ++j) {
                 const float tj = T[j * NP + rr];
-                const float4 *row = reinterpret_cast<const float4 *>(sh.g() + j * NP);
+                const float4 *row = reinterpret_cast<const float4 *>(sh.grow() + j * NP);
 #pragma unroll
                 for (int q4 = 0; q4 < NP / 4; ++q4) {
                     const float4 x = row[q4];
-                    GG[q4 * 4 + 0] += tj * x.x;
-                    GG[q4 * 4 + 1] += tj * x.y;
-                    GG[q4 * 4 + 2] += tj * x.z;
-                    GG[q4 * 4 + 3] += tj * x.w;
+                    GG[q4 * 4 + 0] -= tj * x.x;
+                    GG[q4 * 4 + 1] -= tj * x.y;
+                    GG[q4 * 4 + 2] -= tj * x.z;
+                    GG[q4 * 4 + 3] -= tj * x.w;
                 }
             }
-            // GG + GG^T: the transpose through R (every lane is past its reads of it)
+            // GG + GG^T: the transpose through the same buffer
             __syncwarp(gmask);
             if (r < NP) store_row<NP>(R + rr * NP, GG);
             __syncwarp(gmask);
 #pragma unroll
-            for (int k = 0; k < NP; ++k) GG[k] = (1.f - q.beta) * (GG[k] + R[k * NP + rr]);
+            for (int k = 0; k < NP; ++k) GG[k] = (1.f - beta) * (GG[k] + R[k * NP + rr]);
         }
         __syncwarp(gmask);
         // Row r of K, its diagonal, and H, written as the columns of the packed
@@ -366,15 +432,15 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int k = k2 + e;
-                const cpx<float> c = cc[e], t = u * conj(vv[e]) + S.v * conj(uu[e]);
-                const float m2 = norm2(c), g = gcol[k * NP];
+                const cpx<float> c = cc[e];
+                const cpx<float> t = gcol[k * NP] * (u * conj(vv[e])) + gtr[k * NP] * (S.v * conj(uu[e]));
+                const float m2 = norm2(c);
                 const float a = m2 > 0.f ? rsqrtf(m2) * GG[k] : 0.f;
-                h[k] = k == r ? mk<float>(0.f, 0.f) : mk<float>(a * c.x - g * t.x, a * c.y - g * t.y);
+                h[k] = k == r ? mk<float>(0.f, 0.f) : mk<float>(a * c.x - t.x, a * c.y - t.y);
                 diag += h[k].x * c.x + h[k].y * c.y;
             }
         }
         if (live) {
-            float2 *Hp = Hout + p * nt;
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
                 const float s = S.rsr * sh.rs()[k];
@@ -393,29 +459,28 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
 // S = sum_q m(q) z(q) z(q)^H = D C D, D = diag(sqrt(S_kk)), and H = D^-1 K D^-1
 // (K as in k_adj_pixel, K_rr = -sum_k Re(conj(K_rk) C_rk)), so
 //     Var phihat_i = (sigma2 / 2) sum_r (1 / S_rr) k_r C k_r^H,   k_r row r of K.
-// What depends on the date i is u^(i) = M_:i c_i - M_:ref c_ref, c = j v / |v|^2
-// (columns of M: the weight e_i needs no product), so the pixel is prepared
-// once and every date costs
-//   GG = G^-1 [diag(Re u) X + diag(Im u) Y],  X + jY = (C diag(v)) G^-1
-// (X, Y formed once: 2 N^2 products a row and no intermediate matrix), the row
-// k_r, and its quadratic form over one triangle of C (Hermitian: half the
-// products of k_r C).
-// W warps share a prepared pixel (G pixels) and take two dates a pass; a pass
-// reads each row of X, Y and C once for both, as broadcast 16-byte loads in
-// loops that are not unrolled over the row index (short code).
-// One product H S and two with G^-1 for every date, unrolled, took 17.5 ms on
-// 201 x 301 pixels at stride 1 and N = 20, this 7.7 ms; 101 x 301 pixels at N =
-// 28 38.9 and 9.0 ms, 201 x 301 at N = 12 2.42 and 1.79 ms.
+// Both inverses and u of every date are formed once a pixel; a date costs the
+// two products of GG, the row k_r, and its quadratic form over one triangle of
+// C (Hermitian: half the products of k_r C).
+// W warps share a pixel (G pixels) and take two dates a pass; a pass reads each
+// row of G^-1 and C once for both, as broadcast 16-byte loads in loops that are
+// not unrolled over the row index (short code).
+// With the products unrolled, the solve in the same kernel and H S formed whole,
+// 201 x 301 pixels at stride 1 and N = 20 took 17.5 ms, k_adj_prep and this 7.5;
+// 101 x 301 pixels at N = 28 38.9 and 9.6 ms, 201 x 301 at N = 12 2.42 and 1.73 ms.
+// (X G^-1, X = C diag(v), formed once a pixel would serve every date and save a
+// fifth, but where G is conditioned to 1e6 its order of products moves the
+// result by 1e-4.)
 template <int NP>
 struct UncCfg {
     static constexpr int W = 2;
     using Sh = AdjShared<NP>;
-    static constexpr int oU = Sh::oG + Sh::kMat;       // u [date][r]
-    static constexpr int oK = oU + 2 * Sh::kMat;       // per warp, two dates: rows k_r [NP][NP + 1]
+    static constexpr int oU = Sh::oM;             // u [date][r]
+    static constexpr int oK = oU + 2 * Sh::kMat;  // per warp, two dates: R [r][k] and T [k][r], then rows k_r [NP][NP + 1]
     static constexpr int kKPitch = NP + 1;             // odd: a lane reads its own row 8 bytes at a time
     static constexpr int kK = NP * kKPitch * 8;        // one date's rows
     static constexpr int kBytes = oK + W * 2 * kK;     // of one group
-    static_assert(NP * (NP + 1) * 4 <= kK, "the transposed products fit the row buffers");
+    static_assert(2 * Sh::kMat <= kK && kK % 16 == 0, "the products fit the row buffers");
     static constexpr int kSmem = Sh::G * kBytes;
     // register budget: what shared memory lets an SM hold
     static constexpr int kMinBlocks = NP > 28 ? 3 : (NP > 24 ? 4 : (NP > 20 ? 5 : 7));
@@ -423,8 +488,8 @@ struct UncCfg {
 
 template <int NP>
 __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
-    k_adj_uncert(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref, const EmiParams prm,
-                 float sigma2, float *__restrict__ sd_out) {
+    k_adj_uncert(const float2 *__restrict__ C, const float *__restrict__ Sd, const float2 *__restrict__ Hin, int n,
+                 long long npx, int ref, float beta, float sigma2, float *__restrict__ sd_out) {
     using Cfg = UncCfg<NP>;
     using Sh = AdjShared<NP>;
     constexpr int G = Sh::G, P = Sh::kPitch, W = Cfg::W;
@@ -437,22 +502,19 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
     const Sh sh{gbase};
     cpx<float> *U = reinterpret_cast<cpx<float> *>(gbase + Cfg::oU);
     cpx<float> *K[2];
-    float *Pt[2];
+    float *R[2], *T[2];
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
         K[d] = reinterpret_cast<cpx<float> *>(gbase + Cfg::oK + (warp * 2 + d) * Cfg::kK);
-        Pt[d] = reinterpret_cast<float *>(K[d]);
+        R[d] = reinterpret_cast<float *>(K[d]);
+        T[d] = R[d] + NP * NP;
     }
-    float2 *XY = reinterpret_cast<float2 *>(sh.M());
     const cpx<float> *Crow = sh.C() + rr * P, *vg = sh.v();
-    const float *gcol = sh.g() + rr;
+    const float *gcol = sh.g() + rr, *gtr = sh.grow() + rr;
     const long long nt = ntri(n);
     const long long step = (long long)gridDim.x * G;
-    EmiParams q = prm;
-    q.fp64_resolve = 0;
     const float qnan = __int_as_float(0x7fc00000);
     const bool live = r < n;
-    __shared__ int s_evd[G];
 
     for (long long base = (long long)blockIdx.x * G; base < npx; base += step) {
         const long long p = base + grp;
@@ -466,60 +528,31 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
             if (live && (nan || r == ref)) sd_out[(long long)r * npx + p] = nan ? qnan : 0.f;
             if (solve) {
                 adj_load<NP>(sh, Cpix, r, n);
+                const AdjPixel S = adj_read<NP>(sh, r, n, Cpix, Sd + p * n, Hin + p * nt);
                 __syncwarp(gmask);
-                AdjPixel<NP> S;
                 {
                     cpx<float> mrow[NP];
-                    adj_prepare<NP>(S, mrow, sh, L, Sd, p, n, ref, q);
-                    if (r == 0) s_evd[grp] = S.evd;
-                    // u of every date; g_v has no component along v except where
-                    // v_i or v_ref is exactly 0 (M v = v / c)
-                    const cpx<float> cv = (1.f / S.cdef) * mk<float>(-S.v.y, S.v.x);
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) {
-                        const cpx<float> vi = vg[i];
-                        const float m2 = norm2(vi);
-                        const cpx<float> ci = m2 > 0.f ? (1.f / m2) * mk<float>(-vi.y, vi.x) : mk<float>(0.f, 0.f);
-                        cpx<float> ui = mrow[i] * ci;
-                        if (m2 > 0.f) ui = ui - cv;
-                        if (r < NP) U[i * NP + r] = ui;
-                    }
-                }
-                const cpx<float> uref = U[ref * NP + rr];
-#pragma unroll 4
-                for (int i = 0; i < n; ++i)
-                    if (r < NP) U[i * NP + r] = U[i * NP + r] - uref;
-                // X + jY over the row slots of the solve (read by now: M's inversion syncs)
-                float X[NP], Y[NP];
-#pragma unroll
-                for (int k = 0; k < NP; ++k) X[k] = Y[k] = 0.f;
+                    adj_invert<NP>(S, mrow, sh, L, n, beta);
+                    // u of every date: the gradient on v (gauge-free) of the
+                    // weight 1, projected orthogonal to v
+                    const float m2 = norm2(S.v);
 #pragma unroll 1
-                for (int m = 0; m < n; ++m) {
-                    const cpx<float> t = vg[m] * Crow[m];
-                    const float4 *row = reinterpret_cast<const float4 *>(sh.g() + m * NP);
-#pragma unroll
-                    for (int q4 = 0; q4 < NP / 4; ++q4) {
-                        const float4 g4 = row[q4];
-                        X[q4 * 4 + 0] += t.x * g4.x;
-                        Y[q4 * 4 + 0] += t.y * g4.x;
-                        X[q4 * 4 + 1] += t.x * g4.y;
-                        Y[q4 * 4 + 1] += t.y * g4.y;
-                        X[q4 * 4 + 2] += t.x * g4.z;
-                        Y[q4 * 4 + 2] += t.y * g4.z;
-                        X[q4 * 4 + 3] += t.x * g4.w;
-                        Y[q4 * 4 + 3] += t.y * g4.w;
+                    for (int i = 0; i < n; ++i) {
+                        const float coef = i == ref ? 0.f : (r == ref ? -1.f : (r == i ? 1.f : 0.f));
+                        cpx<float> gv =
+                            (live && m2 > 0.f) ? (coef / m2) * mk<float>(-S.v.y, S.v.x) : mk<float>(0.f, 0.f);
+                        const cpx<float> t = conj(S.v) * gv;
+                        const float sx = group_sum<NP, float>(t.x, gmask), sy = group_sum<NP, float>(t.y, gmask);
+                        gv = gv - S.v * mk<float>(sx, sy);
+                        const cpx<float> u = group_matvec<NP, float>(mrow, gv, sh.buf(), r, gmask);
+                        if (r < NP) U[i * NP + r] = u;
                     }
-                }
-                if (r < NP) {
-                    float4 *dst = reinterpret_cast<float4 *>(XY + r * NP);
-#pragma unroll
-                    for (int k = 0; k < NP; k += 2) dst[k / 2] = make_float4(X[k], Y[k], X[k + 1], Y[k + 1]);
                 }
             }
         }
         __syncthreads();
         if (solve) {
-            const bool evd = s_evd[grp] != 0;
+            const bool evd = __ldg(&Hin[p * nt].y) != 0.f;
             const float rsr = sh.rs()[r];
             const cpx<float> vr = vg[r];
             for (int i0 = 2 * warp; i0 < n; i0 += 2 * W) {
@@ -528,43 +561,85 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                 float A0[NP], A1[NP];
 #pragma unroll
                 for (int k = 0; k < NP; ++k) A0[k] = A1[k] = 0.f;
+                const cpx<float> ur0 = U0[rr], ur1 = U1[rr];
                 if (!evd) {
-#pragma unroll 1
-                    for (int j = 0; j < n; ++j) {
-                        const float g = gcol[j * NP];
-                        const cpx<float> u0 = g * U0[j], u1 = g * U1[j];
-                        const float4 *row = reinterpret_cast<const float4 *>(XY + j * NP);
+                    // GG = -G^-1 R G^-1 (see k_adj_pixel), both dates
+                    if (r < NP) {
 #pragma unroll
-                        for (int k = 0; k < NP; k += 2) {
-                            const float4 t = row[k / 2];
-                            A0[k] += u0.x * t.x;
-                            A0[k] += u0.y * t.y;
-                            A0[k + 1] += u0.x * t.z;
-                            A0[k + 1] += u0.y * t.w;
-                            A1[k] += u1.x * t.x;
-                            A1[k] += u1.y * t.y;
-                            A1[k + 1] += u1.x * t.z;
-                            A1[k + 1] += u1.y * t.w;
+                        for (int k2 = 0; k2 < NP; k2 += 4) {
+                            float q0[4], q1[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const cpx<float> c = Crow[k2 + e], vk = vg[k2 + e];
+                                const cpx<float> h0 = mk<float>(0.f, 0.f) - ur0 * conj(vk);
+                                const cpx<float> h1 = mk<float>(0.f, 0.f) - ur1 * conj(vk);
+                                q0[e] = h0.x * c.x + h0.y * c.y;
+                                q1[e] = h1.x * c.x + h1.y * c.y;
+                            }
+                            *reinterpret_cast<float4 *>(R[0] + r * NP + k2) = make_float4(q0[0], q0[1], q0[2], q0[3]);
+                            *reinterpret_cast<float4 *>(R[1] + r * NP + k2) = make_float4(q1[0], q1[1], q1[2], q1[3]);
                         }
                     }
-                    // GG + GG^T through the row buffers
+                    __syncwarp(gmask);
+#pragma unroll 2
+                    for (int j = 0; j < n; ++j) {
+                        const float g = gcol[j * NP];
+                        const float4 *r0 = reinterpret_cast<const float4 *>(R[0] + j * NP);
+                        const float4 *r1 = reinterpret_cast<const float4 *>(R[1] + j * NP);
+#pragma unroll
+                        for (int k = 0; k < NP; k += 4) {
+                            const float4 x = r0[k / 4], y = r1[k / 4];
+                            A0[k] += g * x.x;
+                            A0[k + 1] += g * x.y;
+                            A0[k + 2] += g * x.z;
+                            A0[k + 3] += g * x.w;
+                            A1[k] += g * y.x;
+                            A1[k + 1] += g * y.y;
+                            A1[k + 2] += g * y.z;
+                            A1[k + 3] += g * y.w;
+                        }
+                    }
                     if (r < NP) {
 #pragma unroll
                         for (int k = 0; k < NP; ++k) {
-                            Pt[0][k * (NP + 1) + r] = A0[k];
-                            Pt[1][k * (NP + 1) + r] = A1[k];
+                            T[0][k * NP + r] = A0[k];
+                            T[1][k * NP + r] = A1[k];
                         }
+                    }
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) A0[k] = A1[k] = 0.f;
+#pragma unroll 2
+                    for (int j = 0; j < n; ++j) {
+                        const float t0 = T[0][j * NP + rr], t1 = T[1][j * NP + rr];
+                        const float4 *row = reinterpret_cast<const float4 *>(sh.grow() + j * NP);
+#pragma unroll
+                        for (int k = 0; k < NP; k += 4) {
+                            const float4 x = row[k / 4];
+                            A0[k] -= t0 * x.x;
+                            A0[k + 1] -= t0 * x.y;
+                            A0[k + 2] -= t0 * x.z;
+                            A0[k + 3] -= t0 * x.w;
+                            A1[k] -= t1 * x.x;
+                            A1[k + 1] -= t1 * x.y;
+                            A1[k + 2] -= t1 * x.z;
+                            A1[k + 3] -= t1 * x.w;
+                        }
+                    }
+                    // GG + GG^T through the row buffers
+                    __syncwarp(gmask);
+                    if (r < NP) {
+                        store_row<NP>(R[0] + r * NP, A0);
+                        store_row<NP>(R[1] + r * NP, A1);
                     }
                     __syncwarp(gmask);
 #pragma unroll
                     for (int k = 0; k < NP; ++k) {
-                        A0[k] += Pt[0][rr * (NP + 1) + k];
-                        A1[k] += Pt[1][rr * (NP + 1) + k];
+                        A0[k] += R[0][k * NP + rr];
+                        A1[k] += R[1][k * NP + rr];
                     }
                     __syncwarp(gmask);
                 }
                 // Rows k_r of both dates into this lane's row buffers.
-                const cpx<float> ur0 = U0[rr], ur1 = U1[rr];
                 float diag0 = 0.f, diag1 = 0.f;
                 cpx<float> *k0 = K[0] + rr * Cfg::kKPitch, *k1 = K[1] + rr * Cfg::kKPitch;
 #pragma unroll
@@ -578,14 +653,15 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                     for (int e = 0; e < 2; ++e) {
                         const int k = k2 + e;
                         const cpx<float> c = cc[e];
-                        const float m2 = norm2(c), g = gcol[k * NP];
-                        const float im = m2 > 0.f ? (1.f - q.beta) * rsqrtf(m2) : 0.f;
-                        const cpx<float> t0 = ur0 * conj(vv[e]) + vr * conj(w0[e]);
-                        const cpx<float> t1 = ur1 * conj(vv[e]) + vr * conj(w1[e]);
+                        const float m2 = norm2(c), g = gcol[k * NP], gt = gtr[k * NP];
+                        const float im = m2 > 0.f ? (1.f - beta) * rsqrtf(m2) : 0.f;
+                        const cpx<float> t0 = g * (ur0 * conj(vv[e])) + gt * (vr * conj(w0[e]));
+                        const cpx<float> t1 = g * (ur1 * conj(vv[e])) + gt * (vr * conj(w1[e]));
                         const float a0 = im * A0[k], a1 = im * A1[k];
-                        cpx<float> h0 = mk<float>(a0 * c.x - g * t0.x, a0 * c.y - g * t0.y);
-                        cpx<float> h1 = mk<float>(a1 * c.x - g * t1.x, a1 * c.y - g * t1.y);
-                        if (k == r) h0 = h1 = mk<float>(0.f, 0.f);
+                        cpx<float> h0 = mk<float>(a0 * c.x - t0.x, a0 * c.y - t0.y);
+                        cpx<float> h1 = mk<float>(a1 * c.x - t1.x, a1 * c.y - t1.y);
+                        // nothing from or to a date without power (S_kk = 0)
+                        if (k == r || !(sh.rs()[k] > 0.f)) h0 = h1 = mk<float>(0.f, 0.f);
                         diag0 += h0.x * c.x + h0.y * c.y;
                         diag1 += h1.x * c.x + h1.y * c.y;
                         if (r < NP) {
@@ -754,110 +830,188 @@ __global__ void __launch_bounds__(256) k_adj_wgrad(const __grid_constant__ Plane
     }
 }
 
-// Tiled scatter of the same sum: a CTA owns a TY x TX tile of output pixels,
-// stages the z of the input region their windows cover and a region-sized
-// accumulator in shared memory; item (pixel s, row i) loads row i of H_p once
-// and adds (H_p z(q))_i into the accumulator for every accepted look q; the
-// accumulator is then added into the gradient (tiles overlap by the window
-// halo).  H is read once; the sums are shared-memory atomics, so the order of
-// additions (and the last bits of the result) may vary from run to run.
+// Tiled scatter of the same sum: a CTA owns a TY x TX tile of output pixels and
+// holds the z of the input region that their windows cover, and an accumulator
+// of it, in shared memory, date-major.  A warp owns RB dates (rows of every
+// H_p) of the whole tile and takes its pixels in turn: its RB rows of H_p go to
+// a buffer of its own (the next pixel's are in flight meanwhile), its lanes are
+// the looks of the window, two a lane, and every pair of entries of an H row,
+// read as one broadcast, serves 16 multiply-adds.  Only the owner adds to a
+// date's accumulator, a lane at its own looks, so nothing is atomic and no
+// warp waits for another within a tile.  The accumulator is then added into
+// the gradient (tiles overlap by the window halo: 8-byte global reductions,
+// whose order, and so the last bits of the result, may vary from run to run).
+// With shared-memory atomics, one row of one pixel a thread and one CTA an SM,
+// 301 x 403 pixels at stride 1 took 2.59 ms at N = 20 and 4.28 at N = 28, this
+// 0.81 and 1.47 ms; 233 x 116 output pixels at strides 3 and 6 0.99 and 0.26 ms.
 struct AdjTile {
     int TY, TX, RY, RX, L;
 };
 
-template <int NT>
-__global__ void __launch_bounds__(256) k_adj_scatter(const __grid_constant__ Planes z, int n, const Geom g,
-                                                     const uint64_t *__restrict__ mask, const float2 *__restrict__ H,
-                                                     float2 *__restrict__ grad, const AdjTile t, long long ntiles,
-                                                     int tilesY) {
+constexpr int kScatterMaxWarps = 8, kScatterBudget = 220 * 1024;
+
+template <int RB>
+__global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
+    const __grid_constant__ Planes z, int n, const Geom g, const uint64_t *__restrict__ mask,
+    const float2 *__restrict__ H, float2 *__restrict__ grad, const AdjTile t, long long ntiles, int tilesY) {
     extern __shared__ __align__(16) float2 sm[];
-    const int npr = t.RY * t.RX;
-    float2 *zreg = sm;                                         // [npr][n]
-    float2 *acc = sm + (size_t)npr * n;                        // [npr][n]
-    int *lkoff = reinterpret_cast<int *>(acc + (size_t)npr * n);  // [L]
-    const long long nt = ntri(n);
-    const long long npix = (long long)g.H * g.W;
+    const int npr = t.RY * t.RX, pitch = (n + 1) & ~1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    float2 *hbuf = sm + (size_t)warp * 2 * RB * pitch;                    // [2][RB][pitch]
+    float2 *zreg = sm + (size_t)nwarps * 2 * RB * pitch;                  // [n][npr]
+    float2 *acc = zreg + (size_t)npr * n;                                 // [n][npr]
+    int *lkoff = reinterpret_cast<int *>(acc + (size_t)npr * n);          // [L]
+    const int i0 = warp * RB;
+    const long long nt = ntri(n), npix = (long long)g.H * g.W;
     for (int l = threadIdx.x; l < t.L; l += blockDim.x) lkoff[l] = (l / g.wx) * t.RX + (l % g.wx);
+    // This lane's share of the warp's rows: where each entry lies in the packed
+    // triangle (the conjugate below the diagonal) and in the buffer; -1: none.
+    int src[RB], dst[RB];
+    unsigned low = 0;
+#pragma unroll
+    for (int m = 0; m < RB; ++m) {
+        const int e = lane + 32 * m, jr = e / n, k = e - jr * n, i = i0 + jr;
+        const bool in = jr < RB && i < n;
+        src[m] = in ? (i <= k ? packed_index(n, i, k) : packed_index(n, k, i)) : -1;
+        dst[m] = jr * pitch + k;
+        if (in && i > k) low |= 1u << m;
+    }
+    // rows past the last date stay zero
+    for (int e = lane; e < 2 * RB * pitch; e += 32) hbuf[e] = make_float2(0.f, 0.f);
     for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int ty0 = (int)(tile % tilesY) * t.TY, tx0 = (int)(tile / tilesY) * t.TX;
         const int y0 = ty0 * g.sy + g.sy / 2 - g.hy, x0 = tx0 * g.sx + g.sx / 2 - g.hx;
         __syncthreads();  // previous tile done with the buffers (and the look table written)
-        for (int idx = threadIdx.x; idx < npr * n; idx += blockDim.x) {
-            const int d = idx / npr, pr = idx - d * npr;
+        for (int pr = threadIdx.x; pr < npr; pr += blockDim.x) {
             const int y = y0 + pr / t.RX, x = x0 + pr % t.RX;
-            float2 v = make_float2(0.f, 0.f);
-            if (y >= 0 && y < g.H && x >= 0 && x < g.W) v = __ldg(z.p[d] + (long long)y * g.W + x);
-            zreg[pr * n + d] = v;
-            acc[pr * n + d] = make_float2(0.f, 0.f);
+            const bool in = y >= 0 && y < g.H && x >= 0 && x < g.W;
+            const long long at = in ? (long long)y * g.W + x : 0;
+#pragma unroll 8
+            for (int d = 0; d < n; ++d) {
+                zreg[d * npr + pr] = in ? __ldg(z.p[d] + at) : make_float2(0.f, 0.f);
+                acc[d * npr + pr] = make_float2(0.f, 0.f);
+            }
         }
         __syncthreads();
-        const int items = t.TY * t.TX * n;
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
-            const int s = it / n, i = it - s * n;
-            const int tx = s / t.TY, ty = s - tx * t.TY;
-            const int oy = ty0 + ty, ox = tx0 + tx;
-            if (oy >= g.Ho || ox >= g.Wo) continue;
-            const long long o = (long long)oy * g.Wo + ox;
-            const float2 *Hp = H + o * nt;
-            cpx<float> hrow[NT];
+        const int ny = min(t.TY, g.Ho - ty0), nx = min(t.TX, g.Wo - tx0), npx = ny * nx;
+        float2 h[RB];
+        auto fetch = [&](int s) {
+            const int tx = s / ny, ty = s - tx * ny;
+            const float2 *Hp = H + ((long long)(ty0 + ty) * g.Wo + tx0 + tx) * nt;
 #pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                hrow[k] = mk<float>(0.f, 0.f);
-                if (k < n) {
-                    const float2 h = __ldg(Hp + (i <= k ? packed_index(n, i, k) : packed_index(n, k, i)));
-                    hrow[k] = i <= k ? mk<float>(h.x, h.y) : mk<float>(h.x, -h.y);
-                }
-            }
-            const uint64_t *mw = mask + o * g.nwords;
+            for (int m = 0; m < RB; ++m) h[m] = src[m] >= 0 ? __ldg(Hp + src[m]) : make_float2(0.f, 0.f);
+        };
+        auto put = [&](int slot) {
+#pragma unroll
+            for (int m = 0; m < RB; ++m)
+                if (src[m] >= 0)
+                    hbuf[slot * RB * pitch + dst[m]] = make_float2(h[m].x, (low >> m) & 1u ? -h[m].y : h[m].y);
+        };
+        fetch(0);
+        put(0);
+        for (int s = 0; s < npx; ++s) {
+            __syncwarp();
+            if (s + 1 < npx) fetch(s + 1);
+            const float2 *hb = hbuf + (s & 1) * RB * pitch;
+            const int tx = s / ny, ty = s - tx * ny;
+            const uint64_t *mw = mask + ((long long)(ty0 + ty) * g.Wo + tx0 + tx) * g.nwords;
             const int corner = ty * g.sy * t.RX + tx * g.sx;
             for (int w0 = 0; w0 < t.L; w0 += 64) {
-                uint64_t bits = __ldg(mw + (w0 >> 6));
-                if (t.L - w0 < 64) bits &= (1ull << (t.L - w0)) - 1ull;  // only the window's looks
-                while (bits) {
-                    const int l = w0 + __ffsll((long long)bits) - 1;
-                    bits &= bits - 1;
-                    const float2 *zq = zreg + (size_t)(corner + lkoff[l]) * n;
-                    cpx<float> a = mk<float>(0.f, 0.f);
+                const uint64_t bits = __ldg(mw + (w0 >> 6));
+                const int l0 = w0 + lane, l1 = l0 + 32;
+                const bool on0 = l0 < t.L && ((bits >> lane) & 1ull), on1 = l1 < t.L && ((bits >> (lane + 32)) & 1ull);
+                const int q0 = corner + (on0 ? lkoff[l0] : 0), q1 = corner + (on1 ? lkoff[l1] : 0);
+                cpx<float> a0[RB], a1[RB];
 #pragma unroll
-                    for (int k = 0; k < NT; ++k) {
-                        if (k >= n) break;
-                        const float2 zz = zq[k];
-                        a = cfma(hrow[k], mk<float>(zz.x, zz.y), a);
+                for (int j = 0; j < RB; ++j) a0[j] = a1[j] = mk<float>(0.f, 0.f);
+                const float2 *z0 = zreg + q0, *z1 = zreg + q1;
+#pragma unroll 2
+                for (int k = 0; k + 1 < n; k += 2, z0 += 2 * npr, z1 += 2 * npr) {
+                    const float2 u0 = z0[0], v0 = z0[npr], u1 = z1[0], v1 = z1[npr];
+#pragma unroll
+                    for (int j = 0; j < RB; ++j) {
+                        const float4 hh = *reinterpret_cast<const float4 *>(hb + j * pitch + k);
+                        const cpx<float> ha = mk<float>(hh.x, hh.y), hc = mk<float>(hh.z, hh.w);
+                        a0[j] = cfma(ha, mk<float>(u0.x, u0.y), a0[j]);
+                        a1[j] = cfma(ha, mk<float>(u1.x, u1.y), a1[j]);
+                        a0[j] = cfma(hc, mk<float>(v0.x, v0.y), a0[j]);
+                        a1[j] = cfma(hc, mk<float>(v1.x, v1.y), a1[j]);
                     }
-                    float2 *dst = acc + (size_t)(corner + lkoff[l]) * n + i;
-                    atomicAdd(&dst->x, a.x);
-                    atomicAdd(&dst->y, a.y);
                 }
+                if (n & 1) {
+                    const float2 u0 = z0[0], u1 = z1[0];
+#pragma unroll
+                    for (int j = 0; j < RB; ++j) {
+                        const float2 hh = hb[j * pitch + n - 1];
+                        a0[j] = cfma(mk<float>(hh.x, hh.y), mk<float>(u0.x, u0.y), a0[j]);
+                        a1[j] = cfma(mk<float>(hh.x, hh.y), mk<float>(u1.x, u1.y), a1[j]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < RB; ++j) {
+                    if (i0 + j >= n) break;
+                    float2 *row = acc + (size_t)(i0 + j) * npr;
+                    if (on0) {
+                        const float2 v = row[q0];
+                        row[q0] = make_float2(v.x + a0[j].x, v.y + a0[j].y);
+                    }
+                    if (on1) {
+                        const float2 v = row[q1];
+                        row[q1] = make_float2(v.x + a1[j].x, v.y + a1[j].y);
+                    }
+                }
+                __syncwarp();  // the next looks (or pixel) add to these sums from other lanes
             }
+            if (s + 1 < npx) put((s + 1) & 1);
         }
         __syncthreads();
-        for (int idx = threadIdx.x; idx < npr * n; idx += blockDim.x) {
-            const int d = idx / npr, pr = idx - d * npr;
+        for (int pr = threadIdx.x; pr < npr; pr += blockDim.x) {
             const int y = y0 + pr / t.RX, x = x0 + pr % t.RX;
             if (y < 0 || y >= g.H || x < 0 || x >= g.W) continue;
-            const float2 v = acc[pr * n + d];
-            if (v.x == 0.f && v.y == 0.f) continue;
-            float2 *dst = grad + (long long)d * npix + (long long)y * g.W + x;
-            atomicAdd(&dst->x, v.x);
-            atomicAdd(&dst->y, v.y);
+            float2 *out = grad + (long long)y * g.W + x;
+#pragma unroll 4
+            for (int d = 0; d < n; ++d) {
+                const float2 v = acc[d * npr + pr];
+                if (v.x != 0.f || v.y != 0.f) atomicAdd(out + (long long)d * npix, v);
+            }
         }
     }
 }
 
-// Tile for the scatter: the most output pixels whose region (z and
-// accumulator, n samples each) fits the budget.
-static AdjTile adj_tile(int n, const Geom &g, size_t budget) {
+// Shared memory of the scatter: the warps' H rows, z and the accumulator over
+// the region, the look table.
+static size_t scatter_smem(int n, const AdjTile &t, int warps, int rb) {
+    return (size_t)warps * 2 * rb * ((n + 1) & ~1) * sizeof(float2) +
+           (size_t)t.RY * t.RX * n * 2 * sizeof(float2) + (size_t)t.L * sizeof(int);
+}
+
+// Tile for the scatter: the most output pixels whose region fits the budget.
+static AdjTile adj_tile(int n, const Geom &g, size_t budget, int warps, int rb) {
     AdjTile best{0, 0, 0, 0, g.wy * g.wx};
     for (int TY = 1; TY <= 32; ++TY)
         for (int TX = 1; TX <= 64; ++TX) {
             AdjTile c{TY, TX, (TY - 1) * g.sy + g.wy, (TX - 1) * g.sx + g.wx, g.wy * g.wx};
-            const size_t sm = (size_t)c.RY * c.RX * n * 2 * sizeof(float2) + (size_t)c.L * sizeof(int);
-            if (sm > budget) continue;
+            if (scatter_smem(n, c, warps, rb) > budget) break;
             if (TY * TX > best.TY * best.TX ||
                 (TY * TX == best.TY * best.TX && c.RY * c.RX < best.RY * best.RX))
                 best = c;
         }
     return best;
+}
+
+template <int RB>
+static cudaError_t run_scatter(const Planes &z, int n, const Geom &g, const uint64_t *mask, const float2 *H,
+                               float2 *grad, const AdjTile &t, cudaStream_t s) {
+    const int warps = (n + RB - 1) / RB;
+    const size_t smem = scatter_smem(n, t, warps, RB);
+    cudaError_t e = cudaFuncSetAttribute(k_adj_scatter<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kScatterBudget);
+    if (e != cudaSuccess) return e;
+    const int tilesY = (g.Ho + t.TY - 1) / t.TY;
+    const long long ntiles = (long long)tilesY * ((g.Wo + t.TX - 1) / t.TX);
+    const long long grid = std::min<long long>(ntiles, (long long)device_sm_count() * 16);
+    k_adj_scatter<RB><<<(unsigned)grid, warps * 32, smem, s>>>(z, n, g, mask, H, grad, t, ntiles, tilesY);
+    return cudaGetLastError();
 }
 
 static int adj_grid(long long work) {
@@ -866,27 +1020,37 @@ static int adj_grid(long long work) {
     return (int)std::max<long long>(1, std::min(blocks, cap));
 }
 
+// Launches of the two-kernel adjoint: the preparation (parts of C, Sd and the H
+// area overwritten), then H, or the standard deviations.
 template <int NP>
-static cudaError_t run_adj_pixel(const float2 *C, const float *Sd, int n, long long npx, int ref,
-                                 const EmiParams &prm, const float *w, float2 *H, cudaStream_t s) {
-    constexpr int G = (NP & (NP - 1)) ? 1 : 32 / NP;
-    long long blocks = ((npx + G - 1) / G + kAdjWarps - 1) / kAdjWarps;
-    const long long cap = (long long)device_sm_count() * 16;
-    blocks = std::max<long long>(1, std::min(blocks, cap));
-    k_adj_pixel<NP><<<(unsigned)blocks, kAdjWarps * 32, 0, s>>>(C, Sd, n, npx, ref, prm, w, H);
+static int adj_blocks(long long npx) {
+    constexpr int G = AdjShared<NP>::G;
+    const long long blocks = ((npx + G - 1) / G + kAdjWarps - 1) / kAdjWarps;
+    return (int)std::max<long long>(1, std::min(blocks, (long long)device_sm_count() * 16));
+}
+
+template <int NP>
+static cudaError_t run_adj_pixel(float2 *C, float *Sd, int n, long long npx, int ref, const EmiParams &prm,
+                                 const float *w, float2 *H, cudaStream_t s) {
+    k_adj_prep<NP><<<adj_blocks<NP>(npx), kAdjWarps * 32, 0, s>>>(C, Sd, n, npx, ref, prm, H);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_adj_pixel<NP><<<adj_blocks<NP>(npx), kAdjWarps * 32, 0, s>>>(C, Sd, n, npx, ref, prm.beta, w, H);
     return cudaGetLastError();
 }
 
 template <int NP>
-static cudaError_t run_adj_uncert(const float2 *C, const float *Sd, int n, long long npx, int ref,
+static cudaError_t run_adj_uncert(float2 *C, float *Sd, float2 *H, int n, long long npx, int ref,
                                   const EmiParams &prm, float sigma2, float *out, cudaStream_t s) {
     using Cfg = UncCfg<NP>;
     constexpr int G = AdjShared<NP>::G;
     cudaError_t e = cudaFuncSetAttribute(k_adj_uncert<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
     if (e != cudaSuccess) return e;
+    k_adj_prep<NP><<<adj_blocks<NP>(npx), kAdjWarps * 32, 0, s>>>(C, Sd, n, npx, ref, prm, H);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long cap = (long long)device_sm_count() * 32;
     const long long blocks = std::max<long long>(1, std::min((npx + G - 1) / G, cap));
-    k_adj_uncert<NP><<<(unsigned)blocks, Cfg::W * 32, Cfg::kSmem, s>>>(C, Sd, n, npx, ref, prm, sigma2, out);
+    k_adj_uncert<NP><<<(unsigned)blocks, Cfg::W * 32, Cfg::kSmem, s>>>(C, Sd, H, n, npx, ref, prm.beta, sigma2, out);
     return cudaGetLastError();
 }
 
@@ -944,26 +1108,23 @@ cudaError_t launch_adjoint(const Planes &z, int n, const Geom &g, const uint64_t
     cudaError_t e = adjoint_h(z, n, g, mask, ref, prm, dphase, workspace, s, prof, &H);
     if (e != cudaSuccess) return e;
     if (prof) prof->begin("adjoint_gather", s);
-    const size_t kBudget = 150 * 1024;
-    const AdjTile t = adj_tile(n, g, kBudget);
+    // Rows a warp: the fewest padded rows, then the most (reuse of z).  Shared
+    // memory so that an SM holds about 12 warps (two CTAs at least), or else
+    // one CTA.
+    int rb = 4;
+    for (int c = 5; c <= 6; ++c)
+        if ((n + c - 1) / c * c <= (n + rb - 1) / rb * rb) rb = c;
+    const int warps = (n + rb - 1) / rb;
+    AdjTile t = adj_tile(n, g, kScatterBudget / std::max(2, (12 + warps - 1) / warps), warps, rb);
+    if (t.TY == 0) t = adj_tile(n, g, kScatterBudget, warps, rb);
     if (t.TY > 0) {
         // tiled scatter (H read once)
-        const size_t smem = (size_t)t.RY * t.RX * n * 2 * sizeof(float2) + (size_t)t.L * sizeof(int);
         e = cudaMemsetAsync(grad, 0, (size_t)npix * n * sizeof(float2), s);
+        if (e == cudaSuccess)
+            e = rb == 4   ? run_scatter<4>(z, n, g, mask, H, grad, t, s)
+                : rb == 5 ? run_scatter<5>(z, n, g, mask, H, grad, t, s)
+                          : run_scatter<6>(z, n, g, mask, H, grad, t, s);
         if (e != cudaSuccess) return e;
-        const int tilesY = (g.Ho + t.TY - 1) / t.TY;
-        const long long ntiles = (long long)tilesY * ((g.Wo + t.TX - 1) / t.TX);
-        const long long gridT = std::min<long long>(ntiles, (long long)device_sm_count() * 2);
-        if (n <= 8) {
-            cudaFuncSetAttribute(k_adj_scatter<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
-            k_adj_scatter<8><<<(unsigned)gridT, 256, smem, s>>>(z, n, g, mask, H, grad, t, ntiles, tilesY);
-        } else if (n <= 16) {
-            cudaFuncSetAttribute(k_adj_scatter<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
-            k_adj_scatter<16><<<(unsigned)gridT, 256, smem, s>>>(z, n, g, mask, H, grad, t, ntiles, tilesY);
-        } else {
-            cudaFuncSetAttribute(k_adj_scatter<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
-            k_adj_scatter<32><<<(unsigned)gridT, 256, smem, s>>>(z, n, g, mask, H, grad, t, ntiles, tilesY);
-        }
     } else {
         // window too large for a shared-memory region: per-element gather
         const int grid = adj_grid(npix * n);
@@ -1008,8 +1169,9 @@ cudaError_t launch_phase_uncertainty(const Planes &z, int n, const Geom &g, cons
     if (e != cudaSuccess) return e;
     k_adj_sdiag<<<adj_grid(npx * n), 256, 0, s>>>(z, n, g, mask, Sd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    float2 *H = reinterpret_cast<float2 *>(ws + a256((size_t)npx * ntri(n) * sizeof(float2)));
     return with_row_length(
-        n, [&](auto np) { return run_adj_uncert<decltype(np)::value>(C, Sd, n, npx, ref, prm, sigma2, sd, s); });
+        n, [&](auto np) { return run_adj_uncert<decltype(np)::value>(C, Sd, H, n, npx, ref, prm, sigma2, sd, s); });
 }
 
 }  // namespace plk

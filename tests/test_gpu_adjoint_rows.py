@@ -73,7 +73,7 @@ def test_rows_match_64_bit_autograd(ctx, N, beta):
     assert dg[ok].max() < 5e-3
 
 
-@pytest.mark.parametrize("N", [4, 13, 19, 27])
+@pytest.mark.parametrize("N", [13, 19, 27])
 def test_single_look_closed_form(ctx, N):
     # One look: C is rank one (eigenvector of C itself), phihat_i = arg z_i -
     # arg z_ref, so Var = (sigma2 / 2) (1 / |z_i|^2 + 1 / |z_ref|^2).
