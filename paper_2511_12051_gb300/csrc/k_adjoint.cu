@@ -122,6 +122,10 @@ __device__ __forceinline__ void adj_load(const AdjShared<NP> &sh, const float2 *
     if (r < NP) C[NP * P + r] = mk<float>(0.f, 0.f);
 }
 
+// |v|^2 with its one rounding order spelt out, so that both kernels weight the
+// same gradient: where |C| is near singular an ulp of it moves H by 1e-4.
+__device__ __forceinline__ float adj_norm2(cpx<float> v) { return __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)); }
+
 // A prepared pixel (k_adj_prep): this lane's entry of the eigenvector and
 // 1 / sqrt(S_rr) (0 where S_rr = 0), the eigenvalue, and max(1, |lambda|).
 struct AdjPixel {
@@ -338,7 +342,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
             // Gradient on v (gauge-free), projected orthogonal to v.
             const float wr = live ? __ldg(w + (long long)r * npx + p) : 0.f;
             const float wsum = group_sum<NP, float>(live && r != ref ? wr : 0.f, gmask);
-            const float m2 = __fmaf_rn(S.v.x, S.v.x, __fmul_rn(S.v.y, S.v.y));
+            const float m2 = adj_norm2(S.v);
             const float coef = (r == ref) ? -wsum : wr;
             cpx<float> gv = (live && m2 > 0.f) ? (coef / m2) * mk<float>(-S.v.y, S.v.x) : mk<float>(0.f, 0.f);
             const cpx<float> t = conj(S.v) * gv;
@@ -535,7 +539,7 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                     adj_invert<NP>(S, mrow, sh, L, n, beta);
                     // u of every date: the gradient on v (gauge-free) of the
                     // weight 1, projected orthogonal to v
-                    const float m2 = norm2(S.v);
+                    const float m2 = adj_norm2(S.v);
 #pragma unroll 1
                     for (int i = 0; i < n; ++i) {
                         const float coef = i == ref ? 0.f : (r == ref ? -1.f : (r == i ? 1.f : 0.f));
