@@ -399,6 +399,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
 #pragma unroll
                 for (int k = 0; k < NP; ++k) T[k * NP + rr] = GG[k];
             }
+            __syncwarp(gmask);  // lanes past the last row read its column
 #pragma unroll
             for (int k = 0; k < NP; ++k) GG[k] = 0.f;
 #pragma unroll 2
@@ -610,6 +611,7 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                             T[1][k * NP + r] = A1[k];
                         }
                     }
+                    __syncwarp(gmask);  // lanes past the last row read its column
 #pragma unroll
                     for (int k = 0; k < NP; ++k) A0[k] = A1[k] = 0.f;
 #pragma unroll 2
@@ -678,6 +680,7 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                     k0[r] = mk<float>(-diag0, 0.f);
                     k1[r] = mk<float>(-diag1, 0.f);
                 }
+                __syncwarp(gmask);  // lanes past the last row read its K row
                 // k C k^H = Re sum_m conj(k_m) sum_l w_lm k_l C_lm over blocks of
                 // columns m: weight 1 inside the diagonal block (both orders
                 // of a pair appear), 2 below it (one order).
