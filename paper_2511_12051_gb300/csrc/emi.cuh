@@ -62,13 +62,15 @@ __device__ __forceinline__ T group_sum(T v, unsigned gmask) {
     for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(gmask, v, off);
     return v;
 }
-// Largest and smallest of non-negative values (0 for NaN): in single precision
-// one reduction of the bit patterns, which order as the values do, instead of
-// four or five exchanges (a 15-date solve 2% faster).
+// Largest and smallest of non-negative values.  Single precision: one reduction
+// of the bit patterns, which order as the values do, instead of four or five
+// exchanges (a 15-date solve 2% faster); a NaN's pattern lies above infinity's,
+// so the largest is NaN if any value is (a row that is not finite shows however
+// many idle lanes pass 0), and the smallest ignores it.
 template <int NP, class T>
 __device__ __forceinline__ T group_max(T v, unsigned gmask) {
     if constexpr (sizeof(T) == 4) {
-        return __uint_as_float(__reduce_max_sync(gmask, __float_as_uint(fmax(v, T(0)))));
+        return __uint_as_float(__reduce_max_sync(gmask, __float_as_uint(v)));
     } else {
 #pragma unroll
         for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmax(v, __shfl_xor_sync(gmask, v, off));
@@ -78,7 +80,7 @@ __device__ __forceinline__ T group_max(T v, unsigned gmask) {
 template <int NP, class T>
 __device__ __forceinline__ T group_min(T v, unsigned gmask) {
     if constexpr (sizeof(T) == 4) {
-        return __uint_as_float(__reduce_min_sync(gmask, __float_as_uint(fmax(v, T(0)))));
+        return __uint_as_float(__reduce_min_sync(gmask, __float_as_uint(v)));
     } else {
 #pragma unroll
         for (int off = GroupLanes<NP>::value / 2; off >= 1; off >>= 1) v = fmin(v, __shfl_xor_sync(gmask, v, off));

@@ -1,0 +1,51 @@
+"""Coherences and samples that are not finite, or whose squares are not: such a
+pixel is not reported as solved, and has no gradient or uncertainty that looks
+like one."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+SOLVED = (0, 1)   # PLK_PX_EMI, PLK_PX_EMI_FP64
+# every row length filled and not
+NS = [8, 16, 20, 24, 28, 32, 7, 15, 18, 23, 27, 31]
+
+
+@pytest.fixture(scope="module")
+def plk():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2511_12051_gb300 import build, plk as _plk
+    build.build()
+    return _plk
+
+
+def coherences(N, P=40):
+    rng = np.random.default_rng(N)
+    z = rng.standard_normal((P, N, 60)) + 1j * rng.standard_normal((P, N, 60))
+    z = z + 1.2 * (rng.standard_normal((P, 1, 60)) + 1j * rng.standard_normal((P, 1, 60)))
+    S = z @ z.conj().transpose(0, 2, 1)
+    d = 1 / np.sqrt(np.einsum("pii->pi", S).real)
+    i, k = np.triu_indices(N)
+    C = (S * d[:, :, None] * d[:, None, :])[:, i, k].astype(np.complex64)
+    C[:, i == k] = 1
+    return np.ascontiguousarray(C)
+
+
+def link(plk, C, N, fp64_resolve):
+    r = plk.Context("cuda:0").phase_link(torch.from_numpy(C).cuda(), N, 0, plk.default_params(fp64_resolve=fp64_resolve))
+    return r["status"].cpu().numpy(), r["phase"].cpu().numpy()
+
+
+@pytest.mark.parametrize("fp64_resolve", [1, 0])
+@pytest.mark.parametrize("N", NS)
+def test_coherence_beyond_range(plk, N, fp64_resolve):
+    C = coherences(N)
+    want = link(plk, C, N, fp64_resolve)
+    C[1::2, 3] = 1e30   # |c|^2 is infinite in single precision
+    st, ph = link(plk, C, N, fp64_resolve)
+    assert not np.isin(st[1::2], SOLVED).any()
+    # the other pixels of the same warps are left as they are
+    np.testing.assert_array_equal(st[::2], want[0][::2])
+    np.testing.assert_array_equal(ph[:, ::2], want[1][:, ::2])
