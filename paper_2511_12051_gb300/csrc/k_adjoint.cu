@@ -11,7 +11,11 @@
 //   v = unit eigenvector of A for the simple eigenvalue lambda (A = G^-1 o C,
 //     or C itself on the EVD fallback):  dv = -(A - lambda I)^+ dA v, so with
 //     u = (A - lambda I + c v v^H)^-1 (g_v - v v^H g_v)  (u orthogonal to v),
-//     the gradient on A is GA = -u v^H.
+//     the gradient on A is GA = -u v^H.  c has the sign that makes the deflated
+//     matrix definite, so that it is inverted without pivoting: positive where
+//     lambda is the smallest eigenvalue, negative on the fallback, where it is
+//     the largest.  (A single look has C - lambda I + c v v^H = 2 C - N I for
+//     c = lambda, whose leading minor of order N / 2 vanishes.)
 //   A = G^-1 o C:  GC += G^-1 o GA;  R = Re(conj(GA) o C);  GG = -G^-1 R G^-1;
 //     G = (1-beta)|C| + beta I:  GC += (1-beta) GG o C/|C|  (off the diagonal,
 //     which is constant).
@@ -127,7 +131,8 @@ __device__ __forceinline__ void adj_load(const AdjShared<NP> &sh, const float2 *
 __device__ __forceinline__ float adj_norm2(cpx<float> v) { return __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)); }
 
 // A prepared pixel (k_adj_prep): this lane's entry of the eigenvector and
-// 1 / sqrt(S_rr) (0 where S_rr = 0), the eigenvalue, and max(1, |lambda|).
+// 1 / sqrt(S_rr) (0 where S_rr = 0), the eigenvalue, and the deflation's c:
+// max(1, |lambda|), negative on the fallback.
 struct AdjPixel {
     cpx<float> v;
     float rsr, lam, cdef;
@@ -142,7 +147,7 @@ __device__ __forceinline__ AdjPixel adj_read(const AdjShared<NP> &sh, int r, int
     S.rsr = S.live ? Hp[r].x : 0.f;
     S.lam = Cpix[0].x;
     S.evd = Hp[0].y != 0.f;
-    S.cdef = fmaxf(1.f, fabsf(S.lam));
+    S.cdef = S.evd ? -fmaxf(1.f, fabsf(S.lam)) : fmaxf(1.f, fabsf(S.lam));
     sh.v()[r] = S.v;
     sh.rs()[r] = S.rsr;
     return S;
