@@ -728,9 +728,10 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                 const float tr0 = group_sum<NP, float>(s2 > 0.f ? s2 * q0 : 0.f, gmask);
                 const float tr1 = group_sum<NP, float>(s2 > 0.f ? s2 * q1 : 0.f, gmask);
                 if (r == 0) {
-                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = sqrtf(fmaxf(0.5f * sigma2 * tr0, 0.f));
-                    if (i1 != i0 && i1 != ref)
-                        sd_out[(long long)i1 * npx + p] = sqrtf(fmaxf(0.5f * sigma2 * tr1, 0.f));
+                    // a sum rounded below 0 counts as 0, one that is not a number stays so
+                    const float var0 = 0.5f * sigma2 * tr0, var1 = 0.5f * sigma2 * tr1;
+                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = sqrtf(var0 < 0.f ? 0.f : var0);
+                    if (i1 != i0 && i1 != ref) sd_out[(long long)i1 * npx + p] = sqrtf(var1 < 0.f ? 0.f : var1);
                 }
                 __syncwarp(gmask);  // the row buffers are free for the next pass
             }

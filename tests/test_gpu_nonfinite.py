@@ -49,3 +49,14 @@ def test_coherence_beyond_range(plk, N, fp64_resolve):
     # the other pixels of the same warps are left as they are
     np.testing.assert_array_equal(st[::2], want[0][::2])
     np.testing.assert_array_equal(ph[:, ::2], want[1][:, ::2])
+
+
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 13, 16, 20, 24, 28, 32])
+def test_undetermined_phases_are_not_certain(plk, N):
+    # Each date has power at a look of its own: C = I, every vector is an
+    # eigenvector and the phases have no derivative.
+    z = torch.zeros((N, 5, 11), dtype=torch.complex64)
+    z.reshape(N, 55)[range(N), range(N)] = torch.polar(torch.full((N,), 1.5), torch.arange(N) * 0.7)
+    mask = torch.full((1, 1, 1), (1 << 55) - 1, dtype=torch.int64).cuda()
+    sd = plk.Context("cuda:0").phase_uncertainty(z.cuda(), (5, 11, 5, 11), mask, 0, 0.1).cpu()[:, 0, 0]
+    assert sd[0] == 0 and not (sd[1:] < 100).any()   # 0.15 for a coherent pair of such samples
