@@ -145,7 +145,7 @@ __device__ __forceinline__ AdjPixel adj_read(const AdjShared<NP> &sh, int r, int
     S.live = r < n;
     S.v = S.live ? mk<float>(Sdp[r], Cpix[packed_index(n, r, r)].y) : mk<float>(0.f, 0.f);
     S.rsr = S.live ? Hp[r].x : 0.f;
-    S.lam = Cpix[0].x;
+    S.lam = Hp[1].y;
     S.evd = Hp[0].y != 0.f;
     S.cdef = S.evd ? -fmaxf(1.f, fabsf(S.lam)) : fmaxf(1.f, fabsf(S.lam));
     sh.v()[r] = S.v;
@@ -220,11 +220,11 @@ __global__ void __launch_bounds__(256) k_adj_sdiag(const __grid_constant__ Plane
 // depends on the weights.  One kernel of both (110 to 190 KB of code, most of it
 // the solve's) lost a third of its issue slots to instruction fetch.  Per output
 // pixel, in place of what it has read: Sd: Re v;  C: Im v in the imaginary part
-// of the diagonal, lambda = v^H A v (the eigenvalue that the perturbation is
-// about) in the real part of its first entry;  H area: 1 / sqrt(S_kk) (0 where
-// S_kk = 0) in its first n entries, whether the EVD fallback solved the pixel in
-// the first imaginary part.  Pixels without data stay as they are (NaN on C's
-// diagonal).
+// of the diagonal;  H area: 1 / sqrt(S_kk) (0 where S_kk = 0) in its first n
+// entries, whether the EVD fallback solved the pixel in the first imaginary
+// part, lambda = v^H A v (the eigenvalue that the perturbation is about) in the
+// second (n >= 2).  C's diagonal keeps its real part, whose NaN marks a pixel
+// without data: a solve that gives no number is not one, and stays NaN.
 constexpr int kAdjWarps = 2;
 
 template <int NP>
@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
         if (live) {
             const float sr = Sd[p * n + r];
             Sd[p * n + r] = v.x;
-            Hout[p * nt + r] = make_float2(sr > 0.f ? rsqrtf(sr) : 0.f, res.evd ? 1.f : 0.f);
-            Cpix[packed_index(n, r, r)] = make_float2(r == 0 ? lam : 1.f, v.y);
+            Hout[p * nt + r] = make_float2(sr > 0.f ? rsqrtf(sr) : 0.f, r == 1 ? lam : (res.evd ? 1.f : 0.f));
+            Cpix[packed_index(n, r, r)].y = v.y;
         }
         __syncwarp(gmask);
     }
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
         }
         __syncthreads();
         if (solve) {
-            const bool evd = __ldg(&Hin[p * nt].y) != 0.f;
+            const bool evd = __ldg(&Hin[p * nt].y) != 0.f, solved = isfinite(__ldg(&Hin[p * nt + 1].y));
             const float rsr = sh.rs()[r];
             const cpx<float> vr = vg[r];
             for (int i0 = 2 * warp; i0 < n; i0 += 2 * W) {
@@ -730,8 +730,9 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                 if (r == 0) {
                     // a sum rounded below 0 counts as 0, one that is not a number stays so
                     const float var0 = 0.5f * sigma2 * tr0, var1 = 0.5f * sigma2 * tr1;
-                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = sqrtf(var0 < 0.f ? 0.f : var0);
-                    if (i1 != i0 && i1 != ref) sd_out[(long long)i1 * npx + p] = sqrtf(var1 < 0.f ? 0.f : var1);
+                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = !solved ? qnan : sqrtf(var0 < 0.f ? 0.f : var0);
+                    if (i1 != i0 && i1 != ref)
+                        sd_out[(long long)i1 * npx + p] = !solved ? qnan : sqrtf(var1 < 0.f ? 0.f : var1);
                 }
                 __syncwarp(gmask);  // the row buffers are free for the next pass
             }

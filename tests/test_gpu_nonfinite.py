@@ -60,3 +60,22 @@ def test_undetermined_phases_are_not_certain(plk, N):
     mask = torch.full((1, 1, 1), (1 << 55) - 1, dtype=torch.int64).cuda()
     sd = plk.Context("cuda:0").phase_uncertainty(z.cuda(), (5, 11, 5, 11), mask, 0, 0.1).cpu()[:, 0, 0]
     assert sd[0] == 0 and not (sd[1:] < 100).any()   # 0.15 for a coherent pair of such samples
+
+
+@pytest.mark.parametrize("N", [2, 4, 8, 15, 16, 20, 28, 32])
+def test_power_beyond_range_gives_no_gradient(plk, N):
+    # |z|^2 is infinite in the middle window: its pixel has data, but no coherence.
+    ctx, win = plk.Context("cuda:0"), (5, 11, 5, 11)
+    gen = torch.Generator().manual_seed(N)
+    z = torch.randn((N, 5, 33), dtype=torch.complex64, generator=gen) + torch.randn((5, 33), dtype=torch.complex64, generator=gen)
+    z[:, :, 11:22] *= 1e20
+    mask = torch.full((1, 3, 1), (1 << 55) - 1, dtype=torch.int64).cuda()
+    w = torch.randn((N, 1, 3), generator=gen).cuda()
+    bad = torch.zeros(33, dtype=torch.bool)
+    bad[11:22] = True
+    g = ctx.phase_link_backward(z.cuda(), win, mask, 0, w).cpu()
+    assert g[:, :, bad].isnan().all() and g[:, :, ~bad].isfinite().all() and (g[:, :, ~bad] != 0).all()
+    dw = ctx.shp_weight_gradient(z.cuda(), win, mask, 0, w).cpu()[0]
+    assert dw[1].isnan().all() and dw[[0, 2]].isfinite().all()
+    sd = ctx.phase_uncertainty(z.cuda(), win, mask, 0, 0.1).cpu()[:, 0]
+    assert sd[1:, 1].isnan().all() and sd[:, [0, 2]].isfinite().all() and (sd[1:, [0, 2]] > 0).all()
