@@ -25,6 +25,7 @@
 // Per input pixel q and date i (gather):  g_i(q) = sum over the output
 //   pixels p whose window holds q with the mask bit set of (H_p z(q))_i.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "emi.cuh"
@@ -845,21 +846,21 @@ __global__ void __launch_bounds__(256) k_adj_wgrad(const __grid_constant__ Plane
 }
 
 // Tiled scatter of the same sum: a CTA owns a TY x TX tile of output pixels and
-// holds the z of the input region that their windows cover, and an accumulator
+// holds the z of the input region that their windows cover, and accumulators
 // of it, in shared memory, date-major.  A warp owns RB dates (rows of every
-// H_p) of the whole tile and takes its pixels in turn: its RB rows of H_p go to
-// a buffer of its own (the next pixel's are in flight meanwhile), its lanes are
-// the looks of the window, two a lane, and every pair of entries of an H row,
-// read as one broadcast, serves 16 multiply-adds.  Only the owner adds to a
-// date's accumulator, a lane at its own looks, so nothing is atomic and no
-// warp waits for another within a tile.  The accumulator is then added into
-// the gradient (tiles overlap by the window halo: 8-byte global reductions,
-// whose order, and so the last bits of the result, may vary from run to run).
-// With shared-memory atomics, one row of one pixel a thread and one CTA an SM,
-// 301 x 403 pixels at stride 1 took 2.59 ms at N = 20 and 4.28 at N = 28, this
-// 0.81 and 1.47 ms; 233 x 116 output pixels at strides 3 and 6 0.99 and 0.26 ms.
+// H_p) of its team's share of the tile and takes those pixels in turn: its RB
+// rows of H_p go to a buffer of its own (the next pixel's are in flight
+// meanwhile), its lanes are the looks of the window, two a lane, and every pair
+// of entries of an H row, read as one broadcast, serves 16 multiply-adds.  Each
+// team has an accumulator, where only the owner adds to a date's, a lane at its
+// own looks, so nothing is atomic and no warp waits for another within a tile.
+// The teams' sums are then added into the gradient (tiles overlap by the window
+// halo: 8-byte global reductions, whose order, and so the last bits of the
+// result, may vary from run to run).  Few dates need several teams to fill an
+// SM, many dates are warps enough (scatter_plan).  Issue bounds it: 55 of a
+// 5 x 11 window's 64 lane slots work; rejected looks cost as accepted ones.
 struct AdjTile {
-    int TY, TX, RY, RX, L;
+    int TY, TX, RY, RX, L, teams;
 };
 
 constexpr int kScatterMaxWarps = 8, kScatterBudget = 220 * 1024;
@@ -871,11 +872,12 @@ __global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
     extern __shared__ __align__(16) float2 sm[];
     const int npr = t.RY * t.RX, pitch = (n + 1) & ~1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    float2 *hbuf = sm + (size_t)warp * 2 * RB * pitch;                    // [2][RB][pitch]
-    float2 *zreg = sm + (size_t)nwarps * 2 * RB * pitch;                  // [n][npr]
-    float2 *acc = zreg + (size_t)npr * n;                                 // [n][npr]
-    int *lkoff = reinterpret_cast<int *>(acc + (size_t)npr * n);          // [L]
-    const int i0 = warp * RB;
+    const int team = warp % t.teams, i0 = warp / t.teams * RB;
+    float2 *hbuf = sm + (size_t)warp * 2 * RB * pitch;                       // [2][RB][pitch]
+    float2 *zreg = sm + (size_t)nwarps * 2 * RB * pitch;                     // [n][npr]
+    float2 *accs = zreg + (size_t)npr * n;                                   // [teams][n][npr]
+    float2 *acc = accs + (size_t)team * npr * n;                             // this team's
+    int *lkoff = reinterpret_cast<int *>(accs + (size_t)t.teams * npr * n);  // [L]
     const long long nt = ntri(n), npix = (long long)g.H * g.W;
     for (int l = threadIdx.x; l < t.L; l += blockDim.x) lkoff[l] = (l / g.wx) * t.RX + (l % g.wx);
     // This lane's share of the warp's rows: where each entry lies in the packed
@@ -901,11 +903,9 @@ __global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
             const bool in = y >= 0 && y < g.H && x >= 0 && x < g.W;
             const long long at = in ? (long long)y * g.W + x : 0;
 #pragma unroll 8
-            for (int d = 0; d < n; ++d) {
-                zreg[d * npr + pr] = in ? __ldg(z.p[d] + at) : make_float2(0.f, 0.f);
-                acc[d * npr + pr] = make_float2(0.f, 0.f);
-            }
+            for (int d = 0; d < n; ++d) zreg[d * npr + pr] = in ? __ldg(z.p[d] + at) : make_float2(0.f, 0.f);
         }
+        for (int e = threadIdx.x; e < t.teams * n * npr; e += blockDim.x) accs[e] = make_float2(0.f, 0.f);
         __syncthreads();
         const int ny = min(t.TY, g.Ho - ty0), nx = min(t.TX, g.Wo - tx0), npx = ny * nx;
         float2 h[RB];
@@ -921,12 +921,15 @@ __global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
                 if (src[m] >= 0)
                     hbuf[slot * RB * pitch + dst[m]] = make_float2(h[m].x, (low >> m) & 1u ? -h[m].y : h[m].y);
         };
-        fetch(0);
-        put(0);
-        for (int s = 0; s < npx; ++s) {
+        if (team < npx) {
+            fetch(team);
+            put(0);
+        }
+        int slot = 0;
+        for (int s = team; s < npx; s += t.teams, slot ^= 1) {
             __syncwarp();
-            if (s + 1 < npx) fetch(s + 1);
-            const float2 *hb = hbuf + (s & 1) * RB * pitch;
+            if (s + t.teams < npx) fetch(s + t.teams);
+            const float2 *hb = hbuf + slot * RB * pitch;
             const int tx = s / ny, ty = s - tx * ny;
             const uint64_t *mw = mask + ((long long)(ty0 + ty) * g.Wo + tx0 + tx) * g.nwords;
             const int corner = ty * g.sy * t.RX + tx * g.sx;
@@ -976,7 +979,7 @@ __global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
                 }
                 __syncwarp();  // the next looks (or pixel) add to these sums from other lanes
             }
-            if (s + 1 < npx) put((s + 1) & 1);
+            if (s + t.teams < npx) put(slot ^ 1);
         }
         __syncthreads();
         for (int pr = threadIdx.x; pr < npr; pr += blockDim.x) {
@@ -985,30 +988,73 @@ __global__ void __launch_bounds__(kScatterMaxWarps * 32) k_adj_scatter(
             float2 *out = grad + (long long)y * g.W + x;
 #pragma unroll 4
             for (int d = 0; d < n; ++d) {
-                const float2 v = acc[d * npr + pr];
+                float2 v = accs[d * npr + pr];
+                for (int m = 1; m < t.teams; ++m) {
+                    const float2 u = accs[(m * n + d) * npr + pr];
+                    v = make_float2(v.x + u.x, v.y + u.y);
+                }
                 if (v.x != 0.f || v.y != 0.f) atomicAdd(out + (long long)d * npix, v);
             }
         }
     }
 }
 
-// Shared memory of the scatter: the warps' H rows, z and the accumulator over
-// the region, the look table.
+// Shared memory of the scatter: the warps' H rows, z and the teams' accumulators
+// over the region, the look table.
 static size_t scatter_smem(int n, const AdjTile &t, int warps, int rb) {
     return (size_t)warps * 2 * rb * ((n + 1) & ~1) * sizeof(float2) +
-           (size_t)t.RY * t.RX * n * 2 * sizeof(float2) + (size_t)t.L * sizeof(int);
+           (size_t)t.RY * t.RX * n * (1 + t.teams) * sizeof(float2) + (size_t)t.L * sizeof(int);
 }
 
-// Tile for the scatter: the most output pixels whose region fits the budget.
-static AdjTile adj_tile(int n, const Geom &g, size_t budget, int warps, int rb) {
-    AdjTile best{0, 0, 0, 0, g.wy * g.wx};
-    for (int TY = 1; TY <= 32; ++TY)
-        for (int TX = 1; TX <= 64; ++TX) {
-            AdjTile c{TY, TX, (TY - 1) * g.sy + g.wy, (TX - 1) * g.sx + g.wx, g.wy * g.wx};
-            if (scatter_smem(n, c, warps, rb) > budget) break;
-            if (TY * TX > best.TY * best.TX ||
-                (TY * TX == best.TY * best.TX && c.RY * c.RX < best.RY * best.RX))
-                best = c;
+// Tile for the scatter: the most output pixels whose region fits the budget
+// (TY = 0: none does).
+static AdjTile adj_tile(int n, const Geom &g, size_t budget, int warps, int rb, int teams) {
+    AdjTile best{0, 0, 0, 0, g.wy * g.wx, teams};
+    const AdjTile empty{0, 0, 0, 0, g.wy * g.wx, teams};
+    const size_t fixed = scatter_smem(n, empty, warps, rb);
+    if (fixed >= budget) return best;
+    const int region = (int)((budget - fixed) / ((size_t)n * (1 + teams) * sizeof(float2)));
+    for (int TY = 1; TY <= std::min(32, g.Ho); ++TY) {
+        const int RY = (TY - 1) * g.sy + g.wy, RXmax = region / RY;
+        if (RXmax < g.wx) break;
+        const int TX = std::min({64, g.Wo, (RXmax - g.wx) / g.sx + 1}), RX = (TX - 1) * g.sx + g.wx;
+        if (TY * TX > best.TY * best.TX || (TY * TX == best.TY * best.TX && RY * RX < best.RY * best.RX))
+            best = AdjTile{TY, TX, RY, RX, g.wy * g.wx, teams};
+    }
+    return best;
+}
+
+// Teams and tile of the scatter (TY = 0: no tile fits).  More teams and more
+// CTAs an SM put more warps in flight; both shrink the tile, and a small tile
+// spends its time on the region (z in, accumulators cleared and added out).
+// The estimate, in cycles of an SM: a warp takes 1000 + 160 n for 64 looks of a
+// pixel, side by side up to 14 warps an SM, and a region sample costs 0.8 a
+// date and buffer.  Fitted to 136 combinations of 2 to 32 dates, windows of
+// 3 x 3 to 31 x 31, strides and image sizes: the choice is within 10% of the
+// fastest one tried in 121 of them, within 20% in 129.  160 x 240 pixels at
+// stride 1, one team a CTA and this: 13 x 25 windows at N = 4 5.50 and 0.16 ms, at
+// N = 8 2.31 and 0.35, 19 x 39 at N = 4 6.18 and 0.45, 3 x 3 at N = 2 0.33 and 0.05 ms.
+static AdjTile scatter_plan(int n, const Geom &g, int rb) {
+    const int groups = (n + rb - 1) / rb, words = (g.wy * g.wx + 63) / 64, sms = device_sm_count();
+    AdjTile best{};
+    double best_cost = 0.0;
+    for (int teams : {1, 2, 3, 4, 6, 8})
+        for (int ctas : {1, 2, 3, 4, 6, 12}) {
+            const int warps = teams * groups;
+            if (warps > kScatterMaxWarps || warps * ctas > 24) continue;
+            const AdjTile t = adj_tile(n, g, kScatterBudget / ctas, warps, rb, teams);
+            if (t.TY == 0) continue;
+            const double tiles =
+                (double)((g.Ho + t.TY - 1) / t.TY) * ((g.Wo + t.TX - 1) / t.TX) / sms;  // an SM
+            const double side = std::min((double)ctas, std::ceil(tiles));               // of them at a time
+            const double looks = (double)((t.TY * t.TX + teams - 1) / teams) * words * (1000.0 + 160.0 * n);
+            const double cost = std::max(1.0, tiles / ctas) *
+                                (looks * std::max(1.0, warps * side / 14.0) +
+                                 0.8 * n * (2 + teams) * t.RY * t.RX * side);
+            if (best.TY == 0 || cost < best_cost) {
+                best = t;
+                best_cost = cost;
+            }
         }
     return best;
 }
@@ -1016,7 +1062,7 @@ static AdjTile adj_tile(int n, const Geom &g, size_t budget, int warps, int rb) 
 template <int RB>
 static cudaError_t run_scatter(const Planes &z, int n, const Geom &g, const uint64_t *mask, const float2 *H,
                                float2 *grad, const AdjTile &t, cudaStream_t s) {
-    const int warps = (n + RB - 1) / RB;
+    const int warps = t.teams * ((n + RB - 1) / RB);
     const size_t smem = scatter_smem(n, t, warps, RB);
     cudaError_t e = cudaFuncSetAttribute(k_adj_scatter<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kScatterBudget);
@@ -1122,15 +1168,11 @@ cudaError_t launch_adjoint(const Planes &z, int n, const Geom &g, const uint64_t
     cudaError_t e = adjoint_h(z, n, g, mask, ref, prm, dphase, workspace, s, prof, &H);
     if (e != cudaSuccess) return e;
     if (prof) prof->begin("adjoint_gather", s);
-    // Rows a warp: the fewest padded rows, then the most (reuse of z).  Shared
-    // memory so that an SM holds about 12 warps (two CTAs at least), or else
-    // one CTA.
+    // rows a warp: the fewest padded rows, then the most (reuse of z)
     int rb = 4;
     for (int c = 5; c <= 6; ++c)
         if ((n + c - 1) / c * c <= (n + rb - 1) / rb * rb) rb = c;
-    const int warps = (n + rb - 1) / rb;
-    AdjTile t = adj_tile(n, g, kScatterBudget / std::max(2, (12 + warps - 1) / warps), warps, rb);
-    if (t.TY == 0) t = adj_tile(n, g, kScatterBudget, warps, rb);
+    const AdjTile t = scatter_plan(n, g, rb);
     if (t.TY > 0) {
         // tiled scatter (H read once)
         e = cudaMemsetAsync(grad, 0, (size_t)npix * n * sizeof(float2), s);
