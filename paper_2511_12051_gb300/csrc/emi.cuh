@@ -565,7 +565,9 @@ __device__ PixelResult emi_solve(const Loader &load, int r, int n, int ref, cons
     const T norm_g = group_max<NP, T>(live ? rs : T(0), gmask);
     T minpiv = T(1), cond = T(1), norm_gi = T(1);
     bool finite = true;
-    const T pfail = T(kPivotFail), pband = is_fp64 ? T(0) : T(kPivotBand);
+    // Without the re-solve there is no band: the first pivot at or below the
+    // limit itself decides, not one just above it that hides it.
+    const T pfail = T(kPivotFail), pband = (is_fp64 || !prm.fp64_resolve) ? T(0) : T(kPivotBand);
     if (!rank_one) {
         minpiv = gj_invert<NP, T, T, true>(g, rbuf, r, n, gmask, pfail + pband);
         T rsi = 0;
