@@ -408,7 +408,8 @@ __device__ __forceinline__ cpx<T> apply_A(const T (&g)[NP], const Loader &load, 
 // refinement described at emi_solve: reform(mu) rebuilds a[] for a new shift
 // and returns the smallest pivot.  On return d = x^H a x of the last step
 // (1/(lambda - mu) for B^{-1}) and q the last convergence factor measured
-// above the noise floor.  Returns true on convergence.
+// above the noise floor.  Returns true on convergence, false where the product
+// is not finite.
 //
 // floor_num / floor_den (floor_den > 0; 0 = none), a shift below lambda_min(A):
 // when B for the starting shift is not positive definite, the shift lies above
@@ -486,7 +487,7 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
         }
         dl_prev = dl;
         if (dl <= tol2) {
-            converged = true;
+            converged = isfinite(s);  // x also stays where |y|^2 is no number
             break;
         }
         if (in_round < 4 || !((allow_reshift && reshifts < 3) || (stop_slow && !allow_reshift))) continue;

@@ -51,6 +51,14 @@ def test_coherence_beyond_range(plk, N, fp64_resolve):
     np.testing.assert_array_equal(ph[:, ::2], want[1][:, ::2])
 
 
+@pytest.mark.parametrize("fp64_resolve", [1, 0])
+@pytest.mark.parametrize("N", NS)
+def test_coherence_not_a_number(plk, N, fp64_resolve):
+    C = coherences(N)
+    C[1::2, 3] = np.nan
+    assert not np.isin(link(plk, C, N, fp64_resolve)[0][1::2], SOLVED).any()
+
+
 @pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 13, 16, 20, 24, 28, 32])
 def test_undetermined_phases_are_not_certain(plk, N):
     # Each date has power at a look of its own: C = I, every vector is an
