@@ -487,7 +487,7 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
         }
         dl_prev = dl;
         if (dl <= tol2) {
-            converged = isfinite(s);  // x also stays where |y|^2 is no number
+            converged = true;
             break;
         }
         if (in_round < 4 || !((allow_reshift && reshifts < 3) || (stop_slow && !allow_reshift))) continue;
@@ -502,7 +502,9 @@ __device__ __forceinline__ bool inverse_iteration(cpx<T> (&a)[NP], cpx<T> &x, cp
         }
     }
     q = factor();
-    return converged;
+    // x also stays as it is, and counts as converged, where y = a x overflows or
+    // is no number; d, live to the end, shows it (|y|^2, kept for it, cost 0.5%)
+    return converged && isfinite(norm2(d));
 }
 
 // Solve one pixel.  T = float: returns flag = true (and no outputs) for a pixel

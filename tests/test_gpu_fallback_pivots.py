@@ -50,14 +50,15 @@ def test_linked_phases(plk, N, first, fp64_resolve):
     piv[:, :a + 1] = 1
     assert np.all((piv[:, a + 1] > 1.02e-4) & (piv[:, a + 1] < 1.18e-4) & (piv[:, a + 2] < -10))
     lam, V = np.linalg.eigh(F)
-    v = V[:, :, -1] * V[:, :1, -1].conj()
-    want = np.angle(v).T
-    r = plk.Context("cuda:0").phase_link(torch.from_numpy(np.ascontiguousarray(C)).cuda(), N, 0,
+    v = V[:, :, -1]
+    want = np.angle(v * v[:, a, None].conj()).T
+    r = plk.Context("cuda:0").phase_link(torch.from_numpy(np.ascontiguousarray(C)).cuda(), N, a,
                                          plk.default_params(fp64_resolve=fp64_resolve))
     assert np.all(r["status"].cpu().numpy() == 2)
-    ok = (np.abs(v).min(1) > 1e-2) & (lam[:, -1] - lam[:, -2] > 0.2)
-    assert ok.sum() >= 5
-    d = np.angle(np.exp(1j * (r["phase"].cpu().numpy() - want)))[:, ok]
+    # entries whose phase a unit vector's rounding leaves alone: the block's, and others not near 0
+    ok = (np.abs(v) > 1e-2).T & (lam[:, -1] - lam[:, -2] > 0.2)
+    assert ok[a:a + 3].mean() > 0.5
+    d = np.angle(np.exp(1j * (r["phase"].cpu().numpy() - want)))[ok]
     assert np.abs(d).max() <= 1e-4
 
 
