@@ -96,10 +96,6 @@ __device__ __forceinline__ cpx<T> inv_s(cpx<T> a) {
     const T d = T(1) / norm2(a);
     return mk<T>(a.x * d, -a.y * d);
 }
-__device__ __forceinline__ float mul_s(float a, float b) { return a * b; }
-__device__ __forceinline__ double mul_s(double a, double b) { return a * b; }
-template <class T>
-__device__ __forceinline__ cpx<T> mul_s(cpx<T> a, cpx<T> b) { return a * b; }
 __device__ __forceinline__ float fms_s(float a, float b, float c) { return c - a * b; }
 __device__ __forceinline__ double fms_s(double a, double b, double c) { return c - a * b; }
 template <class T>
@@ -340,14 +336,13 @@ __device__ __forceinline__ void load_crow(cpx<T> (&c)[NP], const Loader &load, i
 // unit phasor a lane: row r takes the pairs {r, r + j mod n} for j = 1 ..
 // n / 2 (for even n the last j pairs rows r and r + n/2 twice: rows r < n/2
 // take it), so every lane does n / 2 entries instead of the n - 1 - r that its
-// part of the upper triangle holds, in a loop that is not unrolled.  Unrolled
-// over whole rows, half of them masked, it and the reference phase were 18% of
-// a 15-date solve, and the code (75 KB at 16 entries, 58 KB now) passed the
-// instruction cache.  With the convergence factor formed only where it is
-// looked at and B^{-1} left rotated: 250,007 pixels at N = 15 1.147 -> 0.997
-// ms, 524,288 at N = 17 5.50 -> 4.98 ms, 65,521 at N = 28 1.55 -> 1.45 ms, the
-// linked phases bit for bit the same.  An entry below the diagonal is the
-// conjugate of the pair's term.
+// part of the upper triangle holds, in a loop that is not unrolled: the solve is
+// held by instruction fetch, and unrolled over whole rows, half of them masked,
+// this and the reference phase were 18% of a 15-date solve and 17 of its 75 KB of
+// code.  250,007 pixels at N = 15: k_emi32 1.147 ms unrolled, 0.997 so (together
+// with the convergence factor formed only where it is looked at and B^{-1} left
+// rotated); 524,288 at N = 17 5.50 and 4.98 ms, 65,521 at N = 28 1.55 and 1.45 ms.
+// An entry below the diagonal is the conjugate of the pair's term.
 template <int NP, class T, class Load>
 __device__ __forceinline__ cpx<T> pair_sum(const Load &load, cpx<T> zeta, cpx<T> *buf, int r, int n,
                                            unsigned gmask) {

@@ -228,6 +228,9 @@ __global__ void __launch_bounds__(256) k_adj_sdiag(const __grid_constant__ Plane
 // without data: a solve that gives no number is not one, and stays NaN.
 constexpr int kAdjWarps = 2;
 
+// CTAs an SM that registers are budgeted for: 16 warps at 128 a thread (8 or 7
+// CTAs) for rows of up to 24 entries, 12 at 168 (6 or 5) beyond, the budgets of
+// k_emi32, whose solve this is (at most 48 bytes of spills).
 template <int NP>
 struct AdjMinBlocks {
     static constexpr int value = NP > 24 ? 5 : (NP > 16 ? 7 : 8);
@@ -299,13 +302,12 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
 // -sum_k Re(conj(K_rk) C_rk) / S_rr; K_rk = -g_rk u_r conj(v_k) - g_kr v_r conj(u_k)
 // + (1 - beta) (GG_rk + GG_kr) C_rk / |C_rk|.
 // What bounds it is instruction issue and fetch: a pixel is two eliminations
-// and two products of N x N matrices by one warp.  The products used to be
-// unrolled over both indices, 576 to 1024 multiply-adds of straight-line code
-// each that every warp fetched for itself, in rows of 24 or 32 entries.  As
-// loops over the rows, in rows of 20 to 32 entries in steps of 4, apart from
-// the solve (k_adj_prep), 301 x 403 pixels at stride 1 take 2.55 ms in both
-// kernels instead of 5.36 at N = 20, 5.9 instead of 12.4 at N = 28 and 0.95
-// instead of 1.38 at N = 14.
+// and two products of N x N matrices by one warp.  The products are loops over
+// the rows (unrolled over both indices they are 576 to 1024 multiply-adds of
+// straight-line code each, which every warp fetches for itself), in rows of 20
+// to 32 entries in steps of 4.  301 x 403 pixels at stride 1, this and
+// k_adj_prep: 2.55 ms at N = 20, 5.9 at N = 28 and 0.95 at N = 14; in one kernel,
+// unrolled, in rows of 24 and 32 entries, 5.36, 12.4 and 1.38 ms.
 template <int NP>
 __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
     k_adj_pixel(const float2 *__restrict__ C, const float *__restrict__ Sd, int n, long long npx, int ref,
@@ -493,7 +495,9 @@ struct UncCfg {
     static constexpr int kBytes = oK + W * 2 * kK;     // of one group
     static_assert(2 * Sh::kMat <= kK && kK % 16 == 0, "the products fit the row buffers");
     static constexpr int kSmem = Sh::G * kBytes;
-    // register budget: what shared memory lets an SM hold
+    // CTAs an SM that registers are budgeted for, no more than shared memory
+    // holds (13, 7, 9, 6, 4 and 3 at rows of 8 to 32 entries): 128 registers a
+    // thread at 7, 168 at 5, all 255 at 4 and 3; none spills.
     static constexpr int kMinBlocks = NP > 28 ? 3 : (NP > 24 ? 4 : (NP > 20 ? 5 : 7));
 };
 

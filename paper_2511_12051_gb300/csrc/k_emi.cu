@@ -294,13 +294,6 @@ __global__ void __launch_bounds__(kEmiWarps * 32) k_emi64(const float2 *__restri
     });
 }
 
-// Row source held in registers (indexed with compile-time k after inlining).
-template <int NP, class T>
-struct RegRow {
-    cpx<T> c[NP];
-    __device__ __forceinline__ cpx<T> operator()(int k) const { return c[k]; }
-};
-
 // Double-precision row source in shared memory (one slot per lane): the
 // re-solve reads it to form A and again for the start vector and gamma_t, so
 // it holds no registers in between.
