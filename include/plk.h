@@ -55,8 +55,8 @@ enum {
     PLK_PX_EMI_FP64 = 1,  /* EMI solution re-solved in double precision */
     PLK_PX_EVD = 2,       /* inversion of |C| failed: EVD fallback (Sec. III-B) */
     PLK_PX_NODATA = 3,    /* zero-power centre / empty neighbourhood: NaN outputs */
-    PLK_PX_NOCONV = 4,    /* inverse iteration (EMI or EVD fallback) hit max_iter;
-                             last iterate kept */
+    PLK_PX_NOCONV = 4,    /* inverse iteration (EMI or EVD fallback) hit max_iter
+                             or a product that is not finite; last iterate kept */
     PLK_PX_PS = 5         /* output cell takes the phase of a persistent scatterer
                              (plk_ps_regrid, Supplement "Regridding PS and DS") */
 };
@@ -84,7 +84,8 @@ typedef struct plk_params {
                           a pivot within 2e-5 of the 1e-4 failure limit, are
                           re-solved in double precision; default 1e4 */
     int32_t fp64_resolve; /* 1 (default): re-solve flagged pixels in FP64; 0: keep
-                             the single-precision result */
+                             the single-precision result (|C| fails at the first
+                             pivot at or below the limit) */
     float err_max;     /* pixels whose first-order single-precision error bound
                           (condition of G times |G^-1| times eps over the
                           eigengap seen by the iteration) exceeds err_max are
@@ -425,8 +426,8 @@ plk_status plk_backward_workspace_size(int N, int H, int W, plk_window win, size
  * eigenvalue (it grows as 1 / eigengap); the coherence is recomputed, not
  * stored.  slc [N][H][W]; mask as from plk_shp_select; dphase [N][Ho][Wo];
  * workspace: device memory of plk_backward_workspace_size bytes, owned by
- * the caller (nothing is allocated).  Pixels without data contribute nothing.
- * N <= 32.  Errors: EINVAL (bad argument, small workspace), ECUDA.  The paper
+ * the caller (nothing is allocated).  Pixels without data contribute nothing,
+ * pixels whose solve is not finite NaN.  N <= 32.  Errors: EINVAL (bad argument, small workspace), ECUDA.  The paper
  * states no adjoint. */
 plk_status plk_phase_link_backward(plk_ctx *ctx, const plk_c64 *slc, int N, int H, int W, plk_window win,
                                    const uint64_t *mask, int ref_idx, const plk_params *params,
@@ -439,7 +440,8 @@ plk_status plk_phase_link_backward(plk_ctx *ctx, const plk_c64 *slc, int N, int 
  * weighted sum), evaluated at w = mask: dL/dw_b = (1/2) z(q_b)^H H_p z(q_b),
  * H_p the adjoint's matrix of pixel p (see plk_phase_link_backward).  Samples
  * outside the mask get the derivative of adding them with a small weight;
- * samples outside the image and pixels without data get 0.  Scaling every
+ * samples outside the image and pixels without data get 0, pixels whose solve
+ * is not finite NaN.  Scaling every
  * weight of a pixel leaves its coherence unchanged, so the sum over its
  * masked samples is 0.  dweight [Ho][Wo][wy*wx] float, b = (dy + wy/2) * wx +
  * (dx + wx/2) as in the mask bits.  Workspace as plk_backward_workspace_size.
@@ -455,7 +457,8 @@ plk_status plk_shp_weight_gradient(plk_ctx *ctx, const plk_c64 *slc, int N, int 
  * over the pixel's masked window, Var phihat_i = (sigma2 / 2) sum_q |g(q)|^2 =
  * (sigma2 / 2) tr(H^H H S), S = sum_q m(q) z(q) z(q)^H (the pixel's
  * unnormalised sample covariance); one adjoint solve per date, no window
- * scatter.  phase_std [N][Ho][Wo] float: 0 at ref_idx, NaN without data.
+ * scatter.  phase_std [N][Ho][Wo] float: 0 at ref_idx, NaN without data; NaN at
+ * the other dates where the solve is not finite.
  * Workspace as plk_backward_workspace_size.  Not in the paper (it applies the
  * adjoint to uncertainty propagation).  Errors: EINVAL, EUNSUPPORTED, ECUDA. */
 plk_status plk_phase_uncertainty(plk_ctx *ctx, const plk_c64 *slc, int N, int H, int W, plk_window win,

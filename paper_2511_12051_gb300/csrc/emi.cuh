@@ -336,10 +336,11 @@ __device__ __forceinline__ void load_crow(cpx<T> (&c)[NP], const Loader &load, i
 // unit phasor a lane: row r takes the pairs {r, r + j mod n} for j = 1 ..
 // n / 2 (for even n the last j pairs rows r and r + n/2 twice: rows r < n/2
 // take it), so every lane does n / 2 entries instead of the n - 1 - r that its
-// part of the upper triangle holds, in a loop that is not unrolled: the solve is
-// held by instruction fetch, and unrolled over whole rows, half of them masked,
-// this and the reference phase were 18% of a 15-date solve and 17 of its 75 KB of
-// code.  250,007 pixels at N = 15: k_emi32 1.147 ms unrolled, 0.997 so (together
+// part of the upper triangle holds, in a loop that is not unrolled.  Unrolled over
+// whole rows, half of them masked, this and the reference phase are 18% of a
+// 15-date solve and 17 of 75 KB of code, which then pass the instruction cache
+// (84% hits and 1.08 warps an issue waiting for fetch; 98% and 0.16 so).
+// 250,007 pixels at N = 15: k_emi32 1.147 ms unrolled, 0.997 so (together
 // with the convergence factor formed only where it is looked at and B^{-1} left
 // rotated); 524,288 at N = 17 5.50 and 4.98 ms, 65,521 at N = 28 1.55 and 1.45 ms.
 // An entry below the diagonal is the conjugate of the pair's term.
