@@ -221,11 +221,12 @@ __global__ void __launch_bounds__(256) k_adj_sdiag(const __grid_constant__ Plane
 // depends on the weights.  One kernel of both (110 to 190 KB of code, most of it
 // the solve's) lost a third of its issue slots to instruction fetch.  Per output
 // pixel, in place of what it has read: Sd: Re v;  C: Im v in the imaginary part
-// of the diagonal;  H area: 1 / sqrt(S_kk) (0 where S_kk = 0) in its first n
-// entries, whether the EVD fallback solved the pixel in the first imaginary
-// part, lambda = v^H A v (the eigenvalue that the perturbation is about) in the
-// second (n >= 2).  C's diagonal keeps its real part, whose NaN marks a pixel
-// without data: a solve that gives no number is not one, and stays NaN.
+// of the diagonal;  H area: 1 / sqrt(S_kk) (0 where S_kk = 0, NaN where lambda is
+// not finite) in its first n entries, whether the EVD fallback solved the pixel
+// in the first imaginary part, lambda = v^H A v (the eigenvalue that the
+// perturbation is about) in the second (n >= 2).  C's diagonal keeps its real
+// part, whose NaN marks a pixel without data: a solve that gives no number is
+// not one, and stays NaN.
 constexpr int kAdjWarps = 2;
 
 // CTAs an SM that registers are budgeted for: 16 warps at 128 a thread (8 or 7
@@ -289,7 +290,8 @@ __global__ void __launch_bounds__(kAdjWarps * 32, AdjMinBlocks<NP>::value)
         if (live) {
             const float sr = Sd[p * n + r];
             Sd[p * n + r] = v.x;
-            Hout[p * nt + r] = make_float2(sr > 0.f ? rsqrtf(sr) : 0.f, r == 1 ? lam : (res.evd ? 1.f : 0.f));
+            const float rsr = !isfinite(lam) ? __int_as_float(0x7fc00000) : (sr > 0.f ? rsqrtf(sr) : 0.f);
+            Hout[p * nt + r] = make_float2(rsr, r == 1 ? lam : (res.evd ? 1.f : 0.f));
             Cpix[packed_index(n, r, r)].y = v.y;
         }
         __syncwarp(gmask);
@@ -567,7 +569,7 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
         }
         __syncthreads();
         if (solve) {
-            const bool evd = __ldg(&Hin[p * nt].y) != 0.f, solved = isfinite(__ldg(&Hin[p * nt + 1].y));
+            const bool evd = __ldg(&Hin[p * nt].y) != 0.f;
             const float rsr = sh.rs()[r];
             const cpx<float> vr = vg[r];
             for (int i0 = 2 * warp; i0 < n; i0 += 2 * W) {
@@ -730,14 +732,13 @@ __global__ void __launch_bounds__(UncCfg<NP>::W * 32, UncCfg<NP>::kMinBlocks)
                     }
                 }
                 const float s2 = live ? rsr * rsr : 0.f;
-                const float tr0 = group_sum<NP, float>(s2 > 0.f ? s2 * q0 : 0.f, gmask);
-                const float tr1 = group_sum<NP, float>(s2 > 0.f ? s2 * q1 : 0.f, gmask);
+                const float tr0 = group_sum<NP, float>(s2 != 0.f ? s2 * q0 : 0.f, gmask);
+                const float tr1 = group_sum<NP, float>(s2 != 0.f ? s2 * q1 : 0.f, gmask);
                 if (r == 0) {
                     // a sum rounded below 0 counts as 0, one that is not a number stays so
                     const float var0 = 0.5f * sigma2 * tr0, var1 = 0.5f * sigma2 * tr1;
-                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = !solved ? qnan : sqrtf(var0 < 0.f ? 0.f : var0);
-                    if (i1 != i0 && i1 != ref)
-                        sd_out[(long long)i1 * npx + p] = !solved ? qnan : sqrtf(var1 < 0.f ? 0.f : var1);
+                    if (i0 != ref) sd_out[(long long)i0 * npx + p] = sqrtf(var0 < 0.f ? 0.f : var0);
+                    if (i1 != i0 && i1 != ref) sd_out[(long long)i1 * npx + p] = sqrtf(var1 < 0.f ? 0.f : var1);
                 }
                 __syncwarp(gmask);  // the row buffers are free for the next pass
             }
